@@ -477,6 +477,7 @@ fp_status fem_pic_status(fem_pic_t* ctx, void* stream) {
     FP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 4, s));
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (h & ST_TIMEOUT) {
+        FP_CUDA_TRY(ctx, field_reset_sync(ctx, s));
         ctx->err = "a kernel gave up waiting for its asynchronous copies";
         return FP_ECUDA;
     }

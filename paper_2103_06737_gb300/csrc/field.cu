@@ -10,6 +10,8 @@
 
 #include "async_copy.cuh"
 #include "field.cuh"
+#include "grid_sync.cuh"
+#include "pcg.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -759,9 +761,10 @@ __global__ void k_perm_scatter(const int32_t* __restrict__ perm, const double* _
 }
 
 // ax (Newmark system only, may be null): also A x for the final x, in DOF order, when the
-// mixed solver ran (F->last_fp64[slot] == 0 afterwards); the FP64 solver leaves it alone
+// mixed solver ran (F->last_fp64[slot] == 0 afterwards); the FP64 solver leaves it alone.
+// x_zero: the start is zero whatever x holds.
 fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double tol, const double* scale_vec,
-                  int max_iter, int slot, cudaStream_t s, double* ax = nullptr) {
+                  int max_iter, int slot, cudaStream_t s, double* ax = nullptr, bool x_zero = false) {
     FieldDev* F = ctx->field;
     int use64 = ctx->solver_fp64;
     if (ctx->solver_sys[system] >= 0) use64 = ctx->solver_sys[system] == FP_PC_JACOBI_FP64;
@@ -799,6 +802,21 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
         // the learned preconditioner's BF16 values join the operator in shared memory when
         // the block's slots still fit (8 bytes per slot in all) with the launch co-resident
         if (m.dl16 && m.sm_slots > 0) m.sm_l = F->sm_learned[system];
+        const ResidentPlan& P = F->res[system];
+        if (m.dl16) m.deg = 1;   // the learned preconditioner replaces the polynomial
+        if (P.on && (m.deg <= 1 || P.smem_poly)) {   // on chip: no gather, scatter or clearing launches
+            ResidentArgs a{};
+            a.S = m.S, a.val = m.val, a.val32 = m.val32, a.d16u = reinterpret_cast<const uint16_t*>(m.d16), a.dl16 = m.dl16, a.dinv32 = m.dinv32;
+            a.perm = system == FP_SYS_NEWMARK ? F->perm_e : nullptr;
+            a.n = m.n, a.ns = (int)((m.n + 31) / 32);
+            a.b = rhs, a.x = x, a.px = a.perm ? F->px : x, a.ax = ax, a.x_zero = x_zero;
+            a.scale_vec = scale_vec, a.r64 = m.r64, a.z = m.z, a.d0 = m.d0, a.d1 = m.d1, a.sync = F->sync;
+            a.deg = m.deg, a.theta = m.theta, a.delta = m.delta, a.tol = m.tol, a.inner_tol = m.inner_tol;
+            a.max_iter = m.max_iter, a.max_outer = m.max_outer, a.out = m.out, a.status = m.status, a.lflag = m.lflag;
+            PhaseTimer pt(ctx, ph, s);
+            return resident_solve(ctx, P, a, s);
+        }
+        if (x_zero) FP_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, m.n * sizeof(double), s));
         PhaseTimer pt(ctx, ph, s);
         const int grid = system == FP_SYS_NEWMARK ? F->grid_e : F->grid_n;
         const int bs = system == FP_SYS_NEWMARK ? F->bs_e : F->bs_n;
@@ -819,6 +837,7 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
     } else {
         a.S = Sell{F->sn_ptr, F->sn_w, F->sn_col}, a.val = F->sn_L, a.dinv = F->Ldinv, a.n = F->nn;
     }
+    if (x_zero) FP_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, a.n * sizeof(double), s));
     a.b = rhs, a.x = x, a.r = F->r, a.z = F->z, a.p = F->p, a.q = F->q, a.red = F->red;
     a.tol = tol, a.scale_vec = scale_vec, a.max_iter = max_iter, a.out = F->out + 4 * slot, a.status = ctx->d_status;
     void* args[] = {&a};
@@ -953,17 +972,18 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
             k_gauss_rhs<double><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn,
                                                       F->node_fixed, F->tmp, (const double*)Q_new, F->nn, F->rhs,
                                                       F->qd);
-        FP_CUDA_TRY(ctx, cudaMemsetAsync(F->delta, 0, F->nn * sizeof(double), s));
         FP_CUDA_TRY(ctx, cudaGetLastError());
         fp_status sn = neumann_rhs(ctx, s);
         if (sn != FP_OK) return sn;
     }
     // learned correction of the projection's zero starting point (node graph), with fallback
+    const bool corrected = learned_active(F, FP_SYS_GAUSS) && learned_model(F, FP_SYS_GAUSS) == FP_LEARNED_GUESS;
     if (learned_active(F, FP_SYS_GAUSS)) {
+        FP_CUDA_TRY(ctx, cudaMemsetAsync(F->delta, 0, F->nn * sizeof(double), s));
         fp_status sl = learned_guess(ctx, FP_SYS_GAUSS, F->rhs, F->delta, s);
         if (sl != FP_OK) return sl;
     }
-    st = run_pcg(ctx, FP_SYS_GAUSS, F->rhs, F->delta, tol, F->qd, max_iter, 1, s);
+    st = run_pcg(ctx, FP_SYS_GAUSS, F->rhs, F->delta, tol, F->qd, max_iter, 1, s, nullptr, !corrected);
     if (st != FP_OK) return st;
     {
         PhaseTimer pt(ctx, PH_SOLVE, s);
@@ -979,6 +999,12 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
 
 }  // namespace
 
+// after a wait of the on-chip solver ran out: the words of its grid exchanges start afresh
+cudaError_t field_reset_sync(fem_pic* ctx, cudaStream_t s) {
+    if (!ctx->field || !ctx->field->sync) return cudaSuccess;
+    return cudaMemsetAsync(ctx->field->sync, 0, grid_sync_bytes(ctx->sm_count), s);
+}
+
 void field_free(fem_pic* ctx) {
     FieldDev* F = ctx->field;
     if (!F) return;
@@ -988,7 +1014,7 @@ void field_free(fem_pic* ctx) {
                     F->delta, F->qd, F->red, F->out, F->Av32, F->Adinv32, F->Lv32, F->Ldinv32, F->r32,
                     F->z32, F->p32, F->q32, F->c32, F->s32, F->d32[0], F->d32[1], F->se_d16, F->sn_d16, F->pe_ptr, F->pe_w, F->pe_col, F->perm_e, F->pe_A, F->pe_A32, F->pe_dinv32, F->pb, F->px, F->alpha, F->msum, F->se_ptr, F->se_w, F->se_col, F->sn_ptr, F->sn_w,
                     F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->se_A32, F->sn_L32, F->pe_cb, F->sn_cb,
-                    F->pe_cd, F->sn_cd};
+                    F->pe_cd, F->sn_cd, F->sync, F->res[0].pp, F->res[1].pp};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete F;
@@ -1257,6 +1283,7 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
 #endif
             if (!d16.empty() && st == FP_OK) st = up(ctx, &F->se_d16, d16);
             F->hptr[FP_SYS_NEWMARK] = ptr;
+            F->hwidth[FP_SYS_NEWMARK] = w;
             F->slots_total[FP_SYS_NEWMARK] = (int64_t)scol.size();
             if (st == FP_OK) st = up(ctx, &F->perm_e, *perm);
             if (st == FP_OK) st = up(ctx, &F->pe_ptr, ptr);
@@ -1283,6 +1310,7 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
             const std::vector<int16_t> d16 = offsets16(scol, ptr, w, hc.nn);
             if (!d16.empty() && st == FP_OK) st = up(ctx, &F->sn_d16, d16);
             F->hptr[FP_SYS_GAUSS] = ptr;
+            F->hwidth[FP_SYS_GAUSS] = w;
             F->slots_total[FP_SYS_GAUSS] = (int64_t)scol.size();
         }
         if (st == FP_OK) st = up(ctx, &F->sn_ptr, ptr);
@@ -1384,6 +1412,13 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
 #endif
     if (FP_SMEM_OPERATOR && st == FP_OK) st = residency(FP_SYS_NEWMARK, hc.ne, F->bs_e, F->grid_e);
     if (FP_SMEM_OPERATOR && st == FP_OK) st = residency(FP_SYS_GAUSS, hc.nn, F->bs_n, F->grid_n);
+    for (int sys = 0; sys < 2 && st == FP_OK; ++sys)
+        if (sys == FP_SYS_NEWMARK ? F->se_d16 : F->sn_d16)
+            st = resident_setup(ctx, sys == FP_SYS_NEWMARK ? hc.ne : hc.nn, F->hwidth[sys], &F->res[sys]);
+    if (st == FP_OK) {
+        FP_CUDA_TRY(ctx, cudaMalloc(&F->sync, grid_sync_bytes(ctx->sm_count)));
+        FP_CUDA_TRY(ctx, cudaMemset(F->sync, 0, grid_sync_bytes(ctx->sm_count)));
+    }
     if (st == FP_OK) {
         F->grid = std::max(F->grid_e, F->grid_n);
         FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->red, 9 * (size_t)F->grid * sizeof(double)));
@@ -1559,9 +1594,9 @@ fp_status fem_pic_field_initial(fem_pic_t* ctx, const void* Q, double* E, double
     else
         k_gauss_rhs<double><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn, F->node_fixed,
                                                   F->tmp, (const double*)Q, F->nn, F->rhs, F->qd);
-    FP_CUDA_TRY(ctx, cudaMemsetAsync(F->delta, 0, F->nn * sizeof(double), s));
     fp_status st = neumann_rhs(ctx, s);
-    if (st == FP_OK) st = run_pcg(ctx, FP_SYS_GAUSS, F->rhs, F->delta, tol, F->qd, max_iter, 1, s);
+    if (st == FP_OK)
+        st = run_pcg(ctx, FP_SYS_GAUSS, F->rhs, F->delta, tol, F->qd, max_iter, 1, s, nullptr, true);
     if (st == FP_OK) st = neumann_gauge(ctx, s);
     if (st != FP_OK) return st;
     k_project<<<ge, kBlock, 0, s>>>(ctx->d_edges, F->edge_fixed, F->delta, F->tmp, F->ne, E);

@@ -36,6 +36,15 @@ double jacobi_lambda_max(const std::vector<int32_t>& rp, const std::vector<int32
 
 struct LearnedDev;  // learned correction (learned.cu)
 
+// launch shape of the on-chip mixed solver for one system (pcg_resident.cu)
+struct ResidentPlan {
+    bool on = false;            // a block's share of the FP32 operator fits in shared memory
+    bool one = false;           // one block
+    int grid = 0, threads = 0, spb = 0, pairs_max = 0;   // spb: slices per block
+    size_t smem = 0, smem_poly = 0;   // with Jacobi or the learned correction; with the polynomial (0: does not fit)
+    int32_t* pp = nullptr;      // device: slot pairs before each slice
+};
+
 struct FieldDev {
     double dt = 0, eps = 0, mu = 0;
     int bc = FP_BC_PEC;             // field boundary condition
@@ -82,12 +91,15 @@ struct FieldDev {
     int sm_slots[2] = {0, 0};
     int sm_learned[2] = {0, 0};     // the learned preconditioner's values fit in shared memory too
     std::vector<int32_t> hptr[2];   // host copies of the SELL slice starts (Newmark, Gauss)
+    std::vector<int32_t> hwidth[2]; // and widths
     double* red = nullptr;          // reduction partials
     double* out = nullptr;          // [8] solver outputs (iterations, rr, bb) of the last two solves
     int grid = 0;                   // co-resident blocks (cooperative launch limit)
     int grid_e = 0, grid_n = 0;     // grids of the edge and node systems
     int bs_e = 256, bs_n = 256;     // and their block sizes
     int last_fp64[2] = {0, 0};      // solver used by the last solve in each info slot
+    ResidentPlan res[2];            // on-chip solver, Newmark and Gauss systems
+    void* sync = nullptr;           // words of the on-chip solver's grid exchanges (grid_sync.cuh)
     LearnedDev* learned[2] = {nullptr, nullptr};  // per system (Newmark, Gauss)
     int learned_sys = FP_SYS_NEWMARK;              // system the fem_pic_learned_* calls address
     bool learned_used[2] = {false, false};         // the last solve in each info slot used its network

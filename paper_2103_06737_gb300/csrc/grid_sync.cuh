@@ -1,0 +1,259 @@
+// Grid-wide sums and barriers of the cooperative solvers.
+//
+// A grid barrier is one trip to L2 to arrive and one to see the last arrival, about 1.2 us on
+// 152 blocks; reading every block's partial sum after it is another trip (2.1-2.6 us for such a
+// sum).  Here the sum rides on the arrival: a block adds {its partial as an integer, 1 arrival}
+// to one 64-bit word, and the poll that sees the last arrival reads the total with it (1.5-1.7 us
+// with the block's own reduction).  Integer addition is associative, so the total does not
+// depend on the order of arrival and every block and every run gets the same bits.
+//
+//   bits 0-7 arrivals, 8-15 blocks whose partial does not fit, 16-63 signed sum of the partials
+//   scaled by a power of two that all blocks choose alike from the sum's previous values, so
+//   that the expected total lies near 2^32: partials below 2^39 fit, and a total of at least
+//   2^24 is resolved as finely as a float.  Otherwise (a sum that grew or fell more than that,
+//   a value that is not finite) all blocks see it and add the floats themselves, in block
+//   order, behind a second barrier.
+//
+// Words are never cleared: a block subtracts what the word held at its last exchange.  Two words
+// are used in turn, since a block may arrive at the next exchange before another has read this
+// one; it cannot arrive at the one after.  (Polling one array of all blocks' partials, or a
+// mailbox of partials per block, measured 2.7-5 us: 152 blocks' words per exchange are more
+// traffic than the trip they save.)
+//
+// Every wait is bounded: a block that does not see the others within kGridWaitNs sets ST_TIMEOUT
+// in the status word and leaves (all its threads together); the others follow, and
+// fem_pic_status clears the words.
+#pragma once
+
+#include "async_copy.cuh"
+#include "internal.cuh"
+
+namespace fempic {
+
+constexpr uint64_t kGridWaitNs = 2000000000ull;      // 2 s
+// device memory of one handle's exchanges (zeroed at setup): the words at rest, the words
+// in use (two exchanges; a line each), then the blocks' partials for the sums that
+// are added one by one (two copies of three doubles per block)
+constexpr size_t kGridLine = 128;
+inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * blocks * 3 * 8; }
+
+#ifdef __CUDACC__
+
+struct GridSyncShared {
+    double part64[3][33];
+    float part[2][3][33];        // per-warp partials, by the exchange's parity
+    float tot[2][2];
+    unsigned long long prev[2][2];   // what each word held after this block's last exchange on it
+    int state[2];                // bit 0: a wait ran out, bit 1: add the partials one by one
+};
+
+template <bool ONE>   // ONE: a single block, no exchange through memory
+struct GridSync {
+    char* mem;
+    GridSyncShared* sh;
+    int32_t* status;
+    uint32_t turn;             // exchanges so far
+    int nb, lane, wid, warps;
+
+    __device__ __forceinline__ void init(void* m, GridSyncShared* s, int32_t* st) {
+        mem = static_cast<char*>(m);
+        sh = s;
+        status = st;
+        turn = 0;
+        nb = gridDim.x;
+        lane = threadIdx.x & 31;
+        wid = threadIdx.x >> 5;
+        warps = blockDim.x >> 5;
+        // nothing changes the words at rest before every block's first arrival
+        if (!ONE && threadIdx.x < 4) s->prev[threadIdx.x >> 1][threadIdx.x & 1] =
+            *reinterpret_cast<volatile unsigned long long*>(mem + 8 * threadIdx.x);
+        __syncthreads();
+    }
+    // by one thread at the end of a launch whose waits all ended: the next launch starts here
+    __device__ __forceinline__ void finish() {
+        if constexpr (!ONE)
+            for (int k = 0; k < 4; ++k)
+                *reinterpret_cast<volatile unsigned long long*>(mem + 8 * k) = sh->prev[k >> 1][k & 1];
+    }
+    __device__ __forceinline__ unsigned long long* word(int par) {
+        return reinterpret_cast<unsigned long long*>(mem + kGridLine * (1 + par));
+    }
+    // one thread: adds q[0..NW) to the words of this exchange and waits until every block has;
+    // the words' increments in d.  Makes what the block wrote before (ordered by the block
+    // barrier) visible to the blocks that leave the exchange.
+    template <int NW>
+    __device__ __forceinline__ bool arrive_wait(int par, const unsigned long long (&q)[NW], unsigned long long (&d)[NW]) {
+        unsigned long long* w = word(par);
+        // the last addition releases, the load of that word acquires
+#pragma unroll
+        for (int k = 1; k < NW; ++k)
+            asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(w + k), "l"(q[k]) : "memory");
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(q[0]) : "memory");
+        uint64_t t0 = 0;
+        for (uint32_t spin = 0;; ++spin) {
+            unsigned long long c[NW];
+            bool all = true;
+            // the acquire last: the loads are in flight together (a word whose arrivals are not
+            // complete yet shows it in its own count)
+#pragma unroll
+            for (int k = 1; k < NW; ++k)
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(c[k]) : "l"(w + k) : "memory");
+            asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(c[0]) : "l"(w) : "memory");
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                d[k] = c[k] - sh->prev[par][k];
+                all = all && (int)(d[k] & 255ull) == nb;
+            }
+            if (all) {
+#pragma unroll
+                for (int k = 0; k < NW; ++k) sh->prev[par][k] = c[k];
+                return true;
+            }
+            if ((spin & 1023u) == 1023u) {
+                if (t0 == 0) t0 = global_ns();
+                if (global_ns() - t0 > kGridWaitNs) return false;
+            }
+        }
+    }
+    // power of two that takes a total of about `expect` near 2^32 (0: no expectation)
+    static __device__ __forceinline__ int scale_exp(float expect) {
+        const int e = (int)((__float_as_uint(expect) >> 23) & 0xffu);
+        return expect > 0.f && e > 0 && e < 255 ? min(max(32 - (e - 127), -96), 96) : 0;
+    }
+    static __device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+
+    // grid barrier: what any thread wrote before is visible to every thread after
+    __device__ __forceinline__ bool barrier() {
+        if (ONE) {
+            __syncthreads();
+            return true;
+        }
+        const int par = (int)(turn++ & 1u);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned long long q[1] = {1ull};
+            unsigned long long d[1];
+            const bool ok = arrive_wait<1>(par, q, d);
+            if (!ok) atomicOr(status, ST_TIMEOUT);
+            sh->state[par] = ok ? 0 : 1;
+        }
+        __syncthreads();
+        return sh->state[par] == 0;
+    }
+
+    // v[k] <- sum over the grid, the same bits in every thread; expect[k]: about what the sums
+    // will be (any value, the same in every block; it only decides how fast the sum is).  Also
+    // a grid barrier.
+    template <int NV>
+    __device__ __forceinline__ bool sum(float (&v)[NV], const float (&expect)[NV]) {
+        static_assert(NV <= 2, "two words per exchange");
+        const int par = (int)(turn++ & 1u);
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) sh->part[par][k][wid] = v[k];
+        __syncthreads();
+        if (ONE || wid == 0) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                v[k] = lane < warps ? sh->part[par][k][lane] : 0.f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+            }
+        }
+        if (ONE) return true;
+        float* parts = reinterpret_cast<float*>(mem + 3 * kGridLine + (size_t)par * nb * 24);
+        if (threadIdx.x == 0) {
+            unsigned long long q[NV], d[NV];
+            int e[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                e[k] = scale_exp(expect[k]);
+                const float x = v[k] * pow2(e[k]);
+                const bool fits = fabsf(x) < 549755813888.f;   // 2^39, and finite
+                q[k] = (fits ? (unsigned long long)__float2ll_rn(x) << 16 : 256ull) + 1ull;
+                parts[k * nb + blockIdx.x] = v[k];             // for the sums added one by one
+            }
+            const bool ok = arrive_wait<NV>(par, q, d);
+            bool exact = false;
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const long long t = (long long)d[k] >> 16;
+                exact = exact || ((d[k] >> 8) & 255ull) != 0 || (t < 16777216ll && t > -16777216ll);
+                sh->tot[par][k] = __ll2float_rn(t) * pow2(-e[k]);
+            }
+            if (!ok) atomicOr(status, ST_TIMEOUT);
+            sh->state[par] = ok ? (exact ? 2 : 0) : 1;
+        }
+        __syncthreads();
+        if (sh->state[par] == 2) {   // the same in every block
+            if (wid == 0) {
+                float t[NV];
+#pragma unroll
+                for (int k = 0; k < NV; ++k) t[k] = 0.f;
+                for (int b = lane; b < nb; b += 32)
+#pragma unroll
+                    for (int k = 0; k < NV; ++k) t[k] += __ldcg(parts + k * nb + b);
+#pragma unroll
+                for (int k = 0; k < NV; ++k) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+                    if (lane == 0) sh->tot[par][k] = t[k];
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] = sh->tot[par][k];
+        return sh->state[par] != 1;
+    }
+
+    // FP64 sums of three values (once per refinement), added in block order
+    __device__ __forceinline__ bool sum64(double (&v)[3]) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sh->part64[k][wid] = v[k];
+        __syncthreads();
+        double* parts = reinterpret_cast<double*>(mem + 3 * kGridLine + (size_t)(turn & 1u) * nb * 24);
+        if (wid == 0) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                v[k] = lane < warps ? sh->part64[k][lane] : 0.0;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+                if (!ONE && lane == 0) parts[k * nb + blockIdx.x] = v[k];
+            }
+        }
+        if (!ONE && !barrier()) return false;
+        if (wid == 0) {
+            if (!ONE) {
+                v[0] = v[1] = v[2] = 0.0;
+                for (int b = lane; b < nb; b += 32)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) v[k] += __ldcg(parts + k * nb + b);
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+            }
+            if (lane == 0)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) sh->part64[k][32] = v[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = sh->part64[k][32];
+        __syncthreads();   // part64 has one copy
+        return true;
+    }
+};
+
+#endif
+}  // namespace fempic

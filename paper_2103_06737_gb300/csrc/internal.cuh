@@ -80,6 +80,7 @@ void incidence_csr(const HostComplex& hc, int which, std::vector<int32_t>* row_p
 namespace fempic {
 struct FieldDev;
 void field_free(fem_pic* ctx);
+cudaError_t field_reset_sync(fem_pic* ctx, cudaStream_t s);
 // phases timed by the optional profiler (fem_pic_profile_*)
 enum Phase : int { PH_PREP = 0, PH_FAST = 1, PH_WALK = 2, PH_PUSH64 = 3, PH_CHARGE = 4, PH_SORT = 5,
                    PH_RESID = 6, PH_SOLVE = 7, PH_CG_NEWMARK = 8, PH_CG_GAUSS = 9, PH_LEARNED = 10,
