@@ -26,9 +26,6 @@ constexpr int kBlock = 256;
 // Cooperative solvers: up to 2 co-resident blocks per SM (1 for 1024-thread blocks); the block
 // size is chosen per system from kSolverBlocks at setup.
 constexpr int kSolverPerSm = 2;
-// fraction of the outer threshold an inner solve aims for when that needs less than
-// inner_tol (the FP32 recurrence residual can differ slightly from the FP64 one)
-constexpr double kInnerMargin = 0.2;
 
 __device__ __forceinline__ double as_f64(float x) { return f2d(x); }
 __device__ __forceinline__ double as_f64(double x) { return x; }
@@ -183,439 +180,6 @@ __global__ void __launch_bounds__(BS, BS >= 1024 ? 1 : kSolverPerSm) k_pcg(PcgAr
     }
 }
 
-// ---------------------------------------------------------------- mixed-precision solver
-// Iterative refinement: the residual r = b - A x and its norm are FP64; each correction
-// A c = r / |r| is solved approximately by Jacobi-PCG on FP32 copies of A and of the
-// vectors, with FP32 dot products and grid sums (until its own residual drops by inner_tol,
-// or by less when that already meets the outer tolerance), then x += |r| c in FP64.  FP64
-// work is one product per refinement.  Two grid barriers per inner iteration (A p is
-// carried as q = A z + beta q).
-
-struct MixedArgs {
-    Sell S;
-    const double* val;     // FP64 operator (outer residual)
-    const float* val32;    // FP32 copy (inner solves)
-    const float* dinv32;
-    int64_t n;
-    const double* b;
-    double* x;
-    double* r64;
-    float *r, *z, *p, *q, *c;
-    // Chebyshev preconditioner of degree deg (1: plain Jacobi) on [theta - delta, theta + delta]
-    int deg;
-    float theta, delta;
-    float *s, *d0, *d1;    // its residual and two buffers of its step (deg > 1)
-    // FP32 operator in shared memory: sm_slots > 0 slots per block (values, then int16
-    // column offsets), copied from val32 / d16 at the start of the launch
-    const int16_t* d16;
-    int sm_slots;
-    int64_t slots_total;
-    double* red;
-    double tol;            // outer: ||b - A x|| <= tol ||ref||
-    double inner_tol;      // inner: residual reduction per refinement
-    const double* scale_vec;
-    int max_iter;          // total inner iterations
-    int max_outer;
-    double* out;
-    int32_t* status;
-    // learned preconditioner (null: off): z = D^-1 r + Dl r with Dl on the operator's SELL
-    // pattern, BF16 (replaces the Chebyshev polynomial); with sm_l the block's slots of Dl are
-    // held in shared memory after the operator's; lflag (may be null) is set to 1 when the
-    // solve fell back to Jacobi because r.z was not positive
-    const __nv_bfloat16* dl16;
-    int sm_l;
-    int* lflag;
-};
-
-// This block's rows of the FP32 operator in shared memory (when the launch holds it there).
-struct SmemOp {
-    const float* v;       // values, SELL order, slots [base, base + count) of the global layout
-    const int16_t* d;     // column - row
-    int64_t base;
-    const __nv_bfloat16* l;   // the learned preconditioner's values of the same slots (or null)
-};
-
-// A block's streamed product runs through its rows in steps of BS rows (thread 0 holds each
-// step's first row).  With FP_SELL_PREFETCH = D > 0, thread 0 asks the TMA engine at every step
-// to bring the SELL entries (columns and values) of the step D steps ahead into L2, so that the
-// dependent column -> x gathers of the rows wait on L2 rather than HBM latency.  Rows of a step
-// are whole 32-row slices; a slice's entries are 32 w slots from ptr, so the range is
-// 128-byte aligned.
-#ifndef FP_SELL_PREFETCH
-#define FP_SELL_PREFETCH 1
-#endif
-__device__ __forceinline__ void sell_prefetch(const Sell& S, const void* val, int vbytes, int64_t i, int64_t r1,
-                                              int64_t stride) {
-#if FP_SELL_PREFETCH
-    if (threadIdx.x != 0) return;
-    const int64_t r0 = i + FP_SELL_PREFETCH * stride;
-    if (r0 >= r1) return;
-    const int64_t re = r0 + stride < r1 ? r0 + stride : r1;
-    const int64_t s0 = r0 >> 5, s1 = (re - 1) >> 5;
-    const int64_t k0 = __ldg(S.ptr + s0), k1 = (int64_t)__ldg(S.ptr + s1) + 32 * (int64_t)__ldg(S.w + s1);
-    if (k1 <= k0) return;
-    bulk_prefetch_l2(S.col + k0, (uint32_t)((k1 - k0) * 4));
-    bulk_prefetch_l2(static_cast<const char*>(val) + k0 * vbytes, (uint32_t)((k1 - k0) * vbytes));
-#endif
-}
-
-// row i of the FP32 operator times x: from shared memory (sm_slots > 0) or from the global
-// SELL copy; chunks of CH independent loads (as in sell_row)
-template <int CH>
-__device__ __forceinline__ float row_product32(const MixedArgs& a, const SmemOp& so, const float* __restrict__ x,
-                                               int64_t i) {
-    if (a.sm_slots == 0) return sell_row_any<float, float>(a.S, a.val32, x, i);
-    const int64_t sl = i >> 5;
-    const int64_t base = __ldg(a.S.ptr + sl) - so.base + (i & 31);
-    const int w = __ldg(a.S.w + sl);
-    float s = 0.f;
-    for (int j0 = 0; j0 < w; j0 += CH) {
-        int c[CH];
-        float av[CH], xv[CH];
-#pragma unroll
-        for (int u = 0; u < CH; ++u) {
-            const bool in = j0 + u < w;
-            c[u] = in ? (int)i + so.d[base + 32 * (j0 + u)] : -1;
-            av[u] = in ? so.v[base + 32 * (j0 + u)] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < CH; ++u) xv[u] = c[u] >= 0 ? __ldcg(x + c[u]) : 0.f;
-#pragma unroll
-        for (int u = 0; u < CH; ++u) s += av[u] * xv[u];
-    }
-    return s;
-}
-
-// entries per chunk of the mixed solver's products: 16 where the block size leaves the
-// registers for them (blocks of at most 256 threads: up to 96 registers a thread), else the
-// SELL default
-#ifndef FP_SMALL_BLOCK_CHUNK
-#define FP_SMALL_BLOCK_CHUNK 16
-#endif
-template <int BS>
-struct ProductChunk {
-    static constexpr int value = BS <= 256 ? FP_SMALL_BLOCK_CHUNK : kSellChunk;
-};
-
-// z = P(r) for the rows [t0, r1) of this block, P the Chebyshev polynomial of degree deg in
-// B = D^-1 A applied to f = D^-1 r (three-term recurrence on [theta - delta, theta + delta]):
-//   d_0 = f / theta, z = d_0, s = f;
-//   k = 1..deg-1:  s <- s - B d_{k-1},  d_k = rho_k rho_{k-1} d_{k-1} + (2 rho_k / delta) s,
-//                  z <- z + d_k,  rho_0 = delta / theta,  rho_k = 1 / (2 theta / delta - rho_{k-1}).
-// P is positive on (0, theta + delta] and beyond it up to 2 theta, so PCG with it stays a
-// symmetric positive definite method.  Each step's product needs the previous d of every
-// block: one grid barrier per step, d in two buffers.  z is published by the caller's next
-// grid barrier.
-template <int CH>
-__device__ __forceinline__ void chebyshev_apply(const MixedArgs& a, const SmemOp& so, int64_t t0, int64_t r1,
-                                                int64_t stride, cg::grid_group& g) {
-    const float th = a.theta, de = a.delta, sig = th / de;
-    float rho = 1.f / sig;
-    for (int64_t i = t0; i < r1; i += stride) {
-        const float f = a.dinv32[i] * a.r[i];
-        const float d = f / th;
-        a.d0[i] = d;
-        a.z[i] = d;
-        a.s[i] = f;
-    }
-    float* dc = a.d0;
-    float* dn = a.d1;
-    for (int k = 1; k < a.deg; ++k) {
-        g.sync();
-        const float rn = 1.f / (2.f * sig - rho);
-        const float c1 = rn * rho, c2 = 2.f * rn / de;
-        for (int64_t i = t0; i < r1; i += stride) {
-            if (a.sm_slots == 0) sell_prefetch(a.S, a.val32, 4, i, r1, stride);
-            const float bd = a.dinv32[i] * row_product32<CH>(a, so, dc, i);
-            const float sk = a.s[i] - bd;
-            const float dk = c1 * dc[i] + c2 * sk;
-            a.s[i] = sk;
-            dn[i] = dk;
-            a.z[i] += dk;
-        }
-        rho = rn;
-        float* t = dc;
-        dc = dn;
-        dn = t;
-    }
-}
-
-// z = D^-1 r + Dl r for the rows [t0, r1) of this block (the learned preconditioner); the
-// product needs every block's r: one grid barrier first.  z is published by the caller's
-// next grid barrier.  With rz_rr, r.z and r.r of these rows are added to rz_rr[0], rz_rr[1].
-__device__ __forceinline__ void learned_apply(const MixedArgs& a, const SmemOp& so, int64_t t0, int64_t r1,
-                                              int64_t stride, cg::grid_group& g, float* rz_rr = nullptr) {
-    g.sync();
-    if (so.l) {   // Dl and the column offsets from shared memory
-        for (int64_t i = t0; i < r1; i += stride) {
-            const int64_t sl = i >> 5;
-            const int64_t base = __ldg(a.S.ptr + sl) - so.base + (i & 31);
-            const int w = __ldg(a.S.w + sl);
-            float t = 0.f;
-            for (int j0 = 0; j0 < w; j0 += kSellChunk) {
-                int c[kSellChunk];
-                float lv[kSellChunk], xv[kSellChunk];
-#pragma unroll
-                for (int u = 0; u < kSellChunk; ++u) {
-                    const bool in = j0 + u < w;
-                    c[u] = in ? (int)i + so.d[base + 32 * (j0 + u)] : -1;
-                    lv[u] = in ? __bfloat162float(so.l[base + 32 * (j0 + u)]) : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? __ldcg(a.r + c[u]) : 0.f;
-#pragma unroll
-                for (int u = 0; u < kSellChunk; ++u) t += lv[u] * xv[u];
-            }
-            const float ri = a.r[i], zi = a.dinv32[i] * ri + t;
-            a.z[i] = zi;
-            if (rz_rr) {
-                rz_rr[0] += ri * zi;
-                rz_rr[1] += ri * ri;
-            }
-        }
-        return;
-    }
-    for (int64_t i = t0; i < r1; i += stride) {
-        sell_prefetch(a.S, a.dl16, 2, i, r1, stride);
-        const float ri = a.r[i], zi = a.dinv32[i] * ri + sell_row_any<__nv_bfloat16, float>(a.S, a.dl16, a.r, i);
-        a.z[i] = zi;
-        if (rz_rr) {
-            rz_rr[0] += ri * zi;
-            rz_rr[1] += ri * ri;
-        }
-    }
-}
-
-// Inner CG in the Chronopoulos-Gear form (one grid sum per iteration instead of two)
-#ifndef FP_CG_ONE_SUM
-#define FP_CG_ONE_SUM 0
-#endif
-
-template <int BS>
-__global__ void __launch_bounds__(BS, BS >= 1024 ? 1 : kSolverPerSm) k_pcg_mixed(MixedArgs a) {
-    cg::grid_group g = cg::this_grid();
-    __shared__ double sh[4][BS / 32 + 1];
-    __shared__ float shf[3][BS / 32 + 1];
-    // rows [r0, r1) of this block: contiguous runs of whole 32-row slices, so the columns a
-    // block gathers (neighbouring DOFs) stay within a window that its SM's L1 can hold
-    const int64_t chunk = ((a.n + gridDim.x - 1) / gridDim.x + 31) & ~(int64_t)31;
-    const int64_t r0 = min(a.n, (int64_t)blockIdx.x * chunk), r1 = min(a.n, r0 + chunk);
-    const int64_t stride = BS;
-    const int64_t t0 = r0 + threadIdx.x;
-    // this block's slots of the FP32 operator into shared memory (whole 32-row slices)
-    extern __shared__ __align__(16) unsigned char dsm[];
-    SmemOp so{reinterpret_cast<const float*>(dsm),
-              reinterpret_cast<const int16_t*>(dsm + 4 * (size_t)a.sm_slots), 0,
-              a.sm_l && a.dl16 ? reinterpret_cast<const __nv_bfloat16*>(dsm + 6 * (size_t)a.sm_slots) : nullptr};
-    if (a.sm_slots > 0) {
-        const int64_t ns = (a.n + 31) >> 5, s0 = r0 >> 5, s1 = (r1 + 31) >> 5;
-        const int64_t b0 = r0 < r1 ? __ldg(a.S.ptr + s0) : 0;
-        const int64_t b1 = r0 < r1 ? (s1 < ns ? __ldg(a.S.ptr + s1) : a.slots_total) : 0;
-        so.base = b0;
-        float* v = reinterpret_cast<float*>(dsm);
-        int16_t* d = reinterpret_cast<int16_t*>(dsm + 4 * (size_t)a.sm_slots);
-        __nv_bfloat16* l = so.l ? reinterpret_cast<__nv_bfloat16*>(dsm + 6 * (size_t)a.sm_slots) : nullptr;
-        for (int64_t k = threadIdx.x; k < b1 - b0; k += BS) {
-            v[k] = __ldg(a.val32 + b0 + k);
-            d[k] = __ldg(a.d16 + b0 + k);
-            if (l) l[k] = a.dl16[b0 + k];
-        }
-        __syncthreads();
-    }
-    double* part0 = a.red;                               // 4 FP64 values per block
-    float* part1 = (float*)(a.red + 4 * gridDim.x);      // 3 FP32 values per block
-    float* part2 = part1 + 3 * gridDim.x;                // 2 FP32 values per block
-    int total = 0, outer = 0;
-    double rr64 = 0.0, ref2 = 0.0, thr = 0.0;
-    bool use_l = a.dl16 != nullptr;   // every block takes the same fallback decision (grid sums)
-    if (use_l && a.lflag && blockIdx.x == 0 && threadIdx.x == 0) *a.lflag = 0;
-    for (;;) {
-        // ---- outer residual in FP64: r = b - A x; its norm and the reference norm
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int64_t i = t0; i < r1; i += stride) {
-            const double bi = a.b[i];
-            const double ri = bi - sell_row<double, double>(a.S, a.val, a.x, i);
-            a.r64[i] = ri;
-            a.c[i] = 0.f;
-            v[0] += ri * ri;
-            v[1] += bi * bi;
-            if (a.scale_vec) v[2] += a.scale_vec[i] * a.scale_vec[i];
-        }
-        grid_sum<BS, 4, double>(v, part0, g, sh);
-        rr64 = v[0];
-        if (outer == 0) {
-            ref2 = a.scale_vec ? v[2] : v[1];
-            thr = a.tol * a.tol * ref2;
-        }
-        if (!(rr64 > thr) || total >= a.max_iter || outer >= a.max_outer) break;
-        ++outer;
-        // ---- inner FP32 Jacobi-PCG on A c = r / ||r||: vectors, products, dot products and
-        // their grid sums all in FP32 (an inner solve only has to reduce its residual by
-        // inner_tol; the FP64 outer residual corrects what FP32 loses)
-        const double rnorm = sqrt(rr64), rinv = 1.0 / rnorm;
-        for (int64_t i = t0; i < r1; i += stride) {
-            const float ri = d2f(a.r64[i] * rinv);
-            a.r[i] = ri;
-            a.z[i] = a.dinv32[i] * ri;
-        }
-        if (use_l)
-            learned_apply(a, so, t0, r1, stride, g);
-        else if (a.deg > 1)
-            chebyshev_apply<ProductChunk<BS>::value>(a, so, t0, r1, stride, g);
-        g.sync();
-        float u[3] = {0.f, 0.f, 0.f};  // r.z, p.q, r.r
-        for (int64_t i = t0; i < r1; i += stride) {
-            if (a.sm_slots == 0) sell_prefetch(a.S, a.val32, 4, i, r1, stride);
-            const float w = row_product32<ProductChunk<BS>::value>(a, so, a.z, i);
-            const float zi = a.z[i], ri = a.r[i];
-            a.p[i] = zi;
-            a.q[i] = w;
-            u[0] += ri * zi;
-            u[1] += zi * w;
-            u[2] += ri * ri;
-        }
-        grid_sum<BS, 3, float>(u, part1, g, shf);
-        if (use_l && !(u[0] > 0.f)) {   // the learned operator is not positive on r: Jacobi from here on
-            use_l = false;
-            if (a.lflag && blockIdx.x == 0 && threadIdx.x == 0) *a.lflag = 1;
-            g.sync();
-            continue;                   // c is still 0: the refinement restarts with Jacobi
-        }
-        float rz = u[0], pq = u[1];
-        // the inner solve stops at a reduction of inner_tol, or earlier when a smaller
-        // reduction (with a margin of kInnerMargin) already meets the outer tolerance
-        const double need = kInnerMargin * sqrt(thr / rr64);
-        const float red = (float)(need > a.inner_tol ? need : a.inner_tol);
-        const float ithr = red * red * u[2];
-#if FP_CG_ONE_SUM
-        // Chronopoulos-Gear form: one grid sum per iteration.  After the update of c and r
-        // and z = P(r), w = A z is formed behind a plain grid barrier, then r.z, r.r and z.w
-        // are summed together; beta = (r.z)/(r.z)_old, p.q = z.w - beta (r.z) / alpha_old
-        // (= p.A p), p = z + beta p, q = w + beta q (= A p).  w is kept in s (free between
-        // applications of the preconditioner).
-        float alpha = pq > 0.f ? rz / pq : 0.f;
-        for (;;) {
-            if (!(pq > 0.f) || total >= a.max_iter) break;
-            float v3[3] = {0.f, 0.f, 0.f};  // r.z, r.r, z.w
-            if (use_l) {
-                for (int64_t i = t0; i < r1; i += stride) {
-                    a.c[i] += alpha * a.p[i];
-                    a.r[i] -= alpha * a.q[i];
-                }
-                learned_apply(a, so, t0, r1, stride, g);
-            } else if (a.deg <= 1) {
-                for (int64_t i = t0; i < r1; i += stride) {
-                    a.c[i] += alpha * a.p[i];
-                    const float ri = a.r[i] - alpha * a.q[i];
-                    a.r[i] = ri;
-                    a.z[i] = a.dinv32[i] * ri;
-                }
-            } else {
-                for (int64_t i = t0; i < r1; i += stride) {
-                    a.c[i] += alpha * a.p[i];
-                    a.r[i] -= alpha * a.q[i];
-                }
-                chebyshev_apply<ProductChunk<BS>::value>(a, so, t0, r1, stride, g);
-            }
-            g.sync();   // z of every block before its product
-            for (int64_t i = t0; i < r1; i += stride) {
-                const float zi = a.z[i], ri = a.r[i];
-                const float w = row_product32<ProductChunk<BS>::value>(a, so, a.z, i);
-                a.s[i] = w;
-                v3[0] += ri * zi;
-                v3[1] += ri * ri;
-                v3[2] += zi * w;
-            }
-            grid_sum<BS, 3, float>(v3, part1, g, shf);
-            ++total;
-            if (!(v3[1] > ithr)) break;
-            if (use_l && !(v3[0] > 0.f)) {   // not positive on this r: keep c, Jacobi from here on
-                use_l = false;
-                if (a.lflag && blockIdx.x == 0 && threadIdx.x == 0) *a.lflag = 1;
-                break;
-            }
-            const float beta = v3[0] / rz;
-            pq = v3[2] - beta * v3[0] / alpha;
-            rz = v3[0];
-            alpha = pq > 0.f ? rz / pq : 0.f;
-            for (int64_t i = t0; i < r1; i += stride) {
-                a.p[i] = a.z[i] + beta * a.p[i];
-                a.q[i] = a.s[i] + beta * a.q[i];
-            }
-        }
-#else
-        for (;;) {
-            if (!(pq > 0.f) || total >= a.max_iter) break;
-            const float alpha = rz / pq;
-            float w2[2] = {0.f, 0.f};  // r.z, r.r
-            if (use_l) {
-                // r.z and r.r come with z; c += alpha p waits for the product loop, which
-                // reads p anyway (or for the exit below)
-                for (int64_t i = t0; i < r1; i += stride) a.r[i] -= alpha * a.q[i];
-                learned_apply(a, so, t0, r1, stride, g, w2);
-            } else if (a.deg <= 1) {
-                for (int64_t i = t0; i < r1; i += stride) {
-                    a.c[i] += alpha * a.p[i];
-                    const float ri = a.r[i] - alpha * a.q[i];
-                    const float zi = a.dinv32[i] * ri;
-                    a.r[i] = ri;
-                    a.z[i] = zi;
-                    w2[0] += ri * zi;
-                    w2[1] += ri * ri;
-                }
-            } else {
-                for (int64_t i = t0; i < r1; i += stride) {
-                    a.c[i] += alpha * a.p[i];
-                    a.r[i] -= alpha * a.q[i];
-                }
-                chebyshev_apply<ProductChunk<BS>::value>(a, so, t0, r1, stride, g);
-                for (int64_t i = t0; i < r1; i += stride) {
-                    const float ri = a.r[i];
-                    w2[0] += ri * a.z[i];
-                    w2[1] += ri * ri;
-                }
-            }
-            grid_sum<BS, 2, float>(w2, part2, g, shf);
-            ++total;
-            const bool l_step = use_l;   // this iteration deferred c += alpha p
-            if (!(w2[1] > ithr) || (use_l && !(w2[0] > 0.f))) {
-                if (use_l && !(w2[0] > 0.f)) {   // not positive on this r: keep c, Jacobi from here on
-                    use_l = false;
-                    if (a.lflag && blockIdx.x == 0 && threadIdx.x == 0) *a.lflag = 1;
-                }
-                if (l_step)
-                    for (int64_t i = t0; i < r1; i += stride) a.c[i] += alpha * a.p[i];
-                break;
-            }
-            const float beta = w2[0] / rz;
-            rz = w2[0];
-            float u2[1] = {0.f};
-            for (int64_t i = t0; i < r1; i += stride) {
-                if (a.sm_slots == 0) sell_prefetch(a.S, a.val32, 4, i, r1, stride);
-                const float w = row_product32<ProductChunk<BS>::value>(a, so, a.z, i);
-                if (l_step) a.c[i] += alpha * a.p[i];
-                const float pi = a.z[i] + beta * a.p[i];
-                const float qi = w + beta * a.q[i];
-                a.p[i] = pi;
-                a.q[i] = qi;
-                u2[0] += pi * qi;
-            }
-            grid_sum<BS, 1, float>(u2, part1, g, shf);
-            pq = u2[0];
-        }
-#endif
-        for (int64_t i = t0; i < r1; i += stride) a.x[i] += rnorm * f2d(a.c[i]);
-        g.sync();
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.out[0] = (double)total;
-        a.out[1] = rr64;
-        a.out[2] = ref2;
-        a.out[3] = (double)outer;
-        if (rr64 > thr) atomicOr(a.status, ST_NOCONV);
-    }
-}
-
 // Newmark right-hand side and the extrapolated initial guess 2E^n - E^{n-1}, in two passes
 // so that the SELL pass does two FP64 multiply-adds per stored entry:
 //   u = 2E^n - E^{n-1} (also the guess), v = -dt^2 (E^n / 2 + E^{n-1} / 4)   (per row)
@@ -711,16 +275,13 @@ __global__ void k_faraday(const int32_t* __restrict__ fe, const double* __restri
 }
 
 constexpr int kSolverBlocks[4] = {128, 256, 512, 1024};
-// largest per-block share of an FP32 operator (4-byte values + 2-byte column offsets) that the
-// mixed solver keeps in shared memory
-constexpr size_t kSmemOperatorBytes = 200 * 1024;
 
-void* solver_kernel(int bs, bool fp64) {
+void* solver_kernel(int bs) {
     switch (bs) {
-        case 128: return fp64 ? (void*)k_pcg<128> : (void*)k_pcg_mixed<128>;
-        case 256: return fp64 ? (void*)k_pcg<256> : (void*)k_pcg_mixed<256>;
-        case 1024: return fp64 ? (void*)k_pcg<1024> : (void*)k_pcg_mixed<1024>;
-        default: return fp64 ? (void*)k_pcg<512> : (void*)k_pcg_mixed<512>;
+        case 128: return (void*)k_pcg<128>;
+        case 256: return (void*)k_pcg<256>;
+        case 1024: return (void*)k_pcg<1024>;
+        default: return (void*)k_pcg<512>;
     }
 }
 
@@ -737,29 +298,6 @@ fp_status up(fem_pic* ctx, T** d, const std::vector<T>& h) {
     return FP_OK;
 }
 
-// b and x into the solver's row order (row r is DOF perm[r]), and the solution back
-__global__ void k_perm_gather(const int32_t* __restrict__ perm, const double* __restrict__ b,
-                              const double* __restrict__ x, double* __restrict__ pb, double* __restrict__ px,
-                              int64_t n) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = __ldg(perm + r);
-        pb[r] = __ldg(b + k);
-        px[r] = __ldg(x + k);
-    }
-}
-
-// ... and, when ax is given, A x = b - r from the solve's last FP64 residual r (the mixed
-// solver stops right after computing it for the final x), back in DOF order as well
-__global__ void k_perm_scatter(const int32_t* __restrict__ perm, const double* __restrict__ px,
-                               double* __restrict__ x, const double* __restrict__ pb,
-                               const double* __restrict__ r64, double* __restrict__ ax, int64_t n) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = __ldg(perm + r);
-        x[k] = px[r];
-        if (ax) ax[k] = pb[r] - r64[r];
-    }
-}
-
 // ax (Newmark system only, may be null): also A x for the final x, in DOF order, when the
 // mixed solver ran (F->last_fp64[slot] == 0 afterwards); the FP64 solver leaves it alone.
 // x_zero: the start is zero whatever x holds.
@@ -772,64 +310,42 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
     F->last_fp64[slot] = use64;
     F->slot_sys[slot] = system;
     if (!use64) {
-        MixedArgs m;
-        if (system == FP_SYS_NEWMARK) {   // the solver's own row order (gathered in and scattered out below)
-            m.S = Sell{F->pe_ptr, F->pe_w, F->pe_col, F->pe_cb, F->pe_cd}, m.val = F->pe_A, m.val32 = F->pe_A32,
-            m.dinv32 = F->pe_dinv32, m.n = F->ne;
-        } else {
-            m.S = Sell{F->sn_ptr, F->sn_w, F->sn_col, F->sn_cb, F->sn_cd}, m.val = F->sn_L, m.val32 = F->sn_L32,
-            m.dinv32 = F->Ldinv32, m.n = F->nn;
-        }
-        m.b = rhs, m.x = x, m.r64 = F->q;
-        m.r = F->r32, m.z = F->z32, m.p = F->p32, m.q = F->q32, m.c = F->c32, m.red = F->red;
-        {
-            // Chebyshev interval [b / ratio, b] with b 5% above the Lanczos estimate of lambda_max
-            const double bmax = 1.05 * F->lmax[system], blo = bmax / ctx->poly_ratio[system];
-            m.deg = ctx->poly_deg[system];
-            m.theta = (float)(0.5 * (bmax + blo));
-            m.delta = (float)(0.5 * (bmax - blo));
-            m.s = F->s32, m.d0 = F->d32[0], m.d1 = F->d32[1];
-        }
-        m.tol = tol, m.inner_tol = ctx->inner_tol, m.scale_vec = scale_vec, m.max_iter = max_iter, m.max_outer = 12;
-        m.out = F->out + 4 * slot, m.status = ctx->d_status;
-        m.dl16 = learned_precond(F, system);
-        m.lflag = m.dl16 ? learned_flag(F, system) : nullptr;
-        m.sm_l = 0;
-        void* args[] = {&m};
-        m.d16 = system == FP_SYS_NEWMARK ? F->se_d16 : F->sn_d16;
-        m.sm_slots = F->sm_slots[system];
-        m.slots_total = F->slots_total[system];
-        // the learned preconditioner's BF16 values join the operator in shared memory when
-        // the block's slots still fit (8 bytes per slot in all) with the launch co-resident
-        if (m.dl16 && m.sm_slots > 0) m.sm_l = F->sm_learned[system];
+        const bool nm = system == FP_SYS_NEWMARK;
+        const __nv_bfloat16* dl16 = learned_precond(F, system);
+        int* lflag = dl16 ? learned_flag(F, system) : nullptr;
+        const int deg = dl16 ? 1 : ctx->poly_deg[system];   // the learned preconditioner replaces the polynomial
+        // Chebyshev interval [b / ratio, b] with b 5% above the Lanczos estimate of lambda_max
+        const double bmax = 1.05 * F->lmax[system], blo = bmax / ctx->poly_ratio[system];
+        const float theta = (float)(0.5 * (bmax + blo)), delta = (float)(0.5 * (bmax - blo));
+        const int32_t* perm = nm ? F->perm_e : nullptr;   // the Newmark system has its own row order
+        const int max_outer = 12;
+        PhaseTimer pt(ctx, ph, s);
         const ResidentPlan& P = F->res[system];
-        if (m.dl16) m.deg = 1;   // the learned preconditioner replaces the polynomial
-        if (P.on && (m.deg <= 1 || P.smem_poly)) {   // on chip: no gather, scatter or clearing launches
+        if (P.on && (deg <= 1 || P.smem_poly)) {
             ResidentArgs a{};
-            a.S = m.S, a.val = m.val, a.val32 = m.val32, a.d16u = reinterpret_cast<const uint16_t*>(m.d16), a.dl16 = m.dl16, a.dinv32 = m.dinv32;
-            a.perm = system == FP_SYS_NEWMARK ? F->perm_e : nullptr;
-            a.n = m.n, a.ns = (int)((m.n + 31) / 32);
-            a.b = rhs, a.x = x, a.px = a.perm ? F->px : x, a.ax = ax, a.x_zero = x_zero;
-            a.scale_vec = scale_vec, a.r64 = m.r64, a.z = m.z, a.d0 = m.d0, a.d1 = m.d1, a.sync = F->sync;
-            a.deg = m.deg, a.theta = m.theta, a.delta = m.delta, a.tol = m.tol, a.inner_tol = m.inner_tol;
-            a.max_iter = m.max_iter, a.max_outer = m.max_outer, a.out = m.out, a.status = m.status, a.lflag = m.lflag;
-            PhaseTimer pt(ctx, ph, s);
+            a.S = nm ? Sell{F->pe_ptr, F->pe_w, F->pe_col} : Sell{F->sn_ptr, F->sn_w, F->sn_col};
+            a.val = nm ? F->pe_A : F->sn_L, a.val32 = nm ? F->pe_A32 : F->sn_L32;
+            a.d16u = reinterpret_cast<const uint16_t*>(nm ? F->se_d16 : F->sn_d16);
+            a.dinv32 = nm ? F->pe_dinv32 : F->Ldinv32, a.dl16 = dl16, a.perm = perm;
+            a.n = nm ? F->ne : F->nn, a.ns = (int)((a.n + 31) / 32);
+            a.b = rhs, a.x = x, a.px = perm ? F->px : x, a.ax = ax, a.x_zero = x_zero, a.scale_vec = scale_vec;
+            a.r64 = F->q, a.z = F->z32, a.d0 = F->d32[0], a.d1 = F->d32[1], a.sync = F->sync;
+            a.deg = deg, a.theta = theta, a.delta = delta, a.tol = tol, a.inner_tol = ctx->inner_tol;
+            a.max_iter = max_iter, a.max_outer = max_outer, a.out = F->out + 4 * slot, a.status = ctx->d_status;
+            a.lflag = lflag;
             return resident_solve(ctx, P, a, s);
         }
-        if (x_zero) FP_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, m.n * sizeof(double), s));
-        PhaseTimer pt(ctx, ph, s);
-        const int grid = system == FP_SYS_NEWMARK ? F->grid_e : F->grid_n;
-        const int bs = system == FP_SYS_NEWMARK ? F->bs_e : F->bs_n;
-        const size_t smem = (size_t)m.sm_slots * (m.sm_l ? 8 : 6);
-        if (system == FP_SYS_NEWMARK) {
-            k_perm_gather<<<grid_of(ctx, F->ne), kBlock, 0, s>>>(F->perm_e, rhs, x, F->pb, F->px, F->ne);
-            m.b = F->pb, m.x = F->px;
-        }
-        FP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel(solver_kernel(bs, false), dim3(grid), dim3(bs), args, smem, s));
-        if (system == FP_SYS_NEWMARK)
-            k_perm_scatter<<<grid_of(ctx, F->ne), kBlock, 0, s>>>(F->perm_e, F->px, x, F->pb, F->q, ax, F->ne);
-        FP_CUDA_TRY(ctx, cudaGetLastError());
-        return FP_OK;
+        StreamArgs a{};
+        a.learned = dl16 != nullptr, a.x_zero = x_zero;
+        a.dinv32 = nm ? F->pe_dinv32 : F->Ldinv32, a.perm = perm;
+        a.b = rhs, a.x = x, a.pb = perm ? F->pb : const_cast<double*>(rhs), a.px = perm ? F->px : x, a.ax = ax;
+        a.scale_vec = scale_vec, a.r64 = F->q;
+        a.r = F->r32, a.z = F->z32, a.p = F->p32, a.q = F->q32, a.c = F->c32, a.s = F->s32;
+        a.d0 = F->d32[0], a.d1 = F->d32[1], a.sync = F->sync;
+        a.deg = deg, a.theta = theta, a.delta = delta, a.tol = tol, a.inner_tol = ctx->inner_tol;
+        a.max_iter = max_iter, a.max_outer = max_outer, a.out = F->out + 4 * slot, a.status = ctx->d_status;
+        a.lflag = lflag;
+        return stream_solve(ctx, F->stream[system], a, s);
     }
     PcgArgs a;
     if (system == FP_SYS_NEWMARK) {
@@ -844,7 +360,7 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
     PhaseTimer pt(ctx, ph, s);
     const int grid = system == FP_SYS_NEWMARK ? F->grid_e : F->grid_n;
     const int bs = system == FP_SYS_NEWMARK ? F->bs_e : F->bs_n;
-    FP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel(solver_kernel(bs, true), dim3(grid), dim3(bs), args, 0, s));
+    FP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel(solver_kernel(bs), dim3(grid), dim3(bs), args, 0, s));
     return FP_OK;
 }
 
@@ -1013,10 +529,10 @@ void field_free(fem_pic* ctx) {
                     F->edge_fixed, F->node_fixed, F->face_edges, F->r, F->z, F->p, F->q, F->rhs, F->tmp,
                     F->delta, F->qd, F->red, F->out, F->Av32, F->Adinv32, F->Lv32, F->Ldinv32, F->r32,
                     F->z32, F->p32, F->q32, F->c32, F->s32, F->d32[0], F->d32[1], F->se_d16, F->sn_d16, F->pe_ptr, F->pe_w, F->pe_col, F->perm_e, F->pe_A, F->pe_A32, F->pe_dinv32, F->pb, F->px, F->alpha, F->msum, F->se_ptr, F->se_w, F->se_col, F->sn_ptr, F->sn_w,
-                    F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->se_A32, F->sn_L32, F->pe_cb, F->sn_cb,
-                    F->pe_cd, F->sn_cd, F->sync, F->res[0].pp, F->res[1].pp};
+                    F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->se_A32, F->sn_L32, F->sync, F->res[0].pp, F->res[1].pp};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (StreamPlan& P : F->stream) stream_free(&P);
     delete F;
     ctx->field = nullptr;
 }
@@ -1145,34 +661,6 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
                     }
             return d;
         };
-        // columns as a 32-bit base per slice position plus lane plus a 16-bit offset (Sell::cb,
-        // Sell::cd); false when some offset does not fit.  The base is the middle of the lanes'
-        // col - lane at that position: in an order where the 32 rows of a slice have the same
-        // stencil (consecutive rows, consecutive neighbours) the offsets stay near 0.
-        auto columns16 = [](const std::vector<int32_t>& scol, const std::vector<int32_t>& sptr,
-                            const std::vector<int32_t>& sw, int64_t n, std::vector<int32_t>* cb,
-                            std::vector<int16_t>* cd) {
-            cb->assign(scol.size() / 32, 0);
-            cd->assign(scol.size(), 0);
-            for (size_t sl = 0; sl < sptr.size(); ++sl)
-                for (int64_t j = 0; j < sw[sl]; ++j) {
-                    int64_t lo = INT64_MAX, hi = INT64_MIN;
-                    for (int64_t lane = 0; lane < 32 && 32 * (int64_t)sl + lane < n; ++lane) {
-                        const int64_t v = (int64_t)scol[sptr[sl] + 32 * j + lane] - lane;
-                        lo = std::min(lo, v);
-                        hi = std::max(hi, v);
-                    }
-                    if (lo > hi) continue;   // no row (never computed)
-                    const int64_t base = lo + (hi - lo) / 2;
-                    if (hi - base > 32767 || lo - base < -32768) return false;
-                    (*cb)[sptr[sl] / 32 + j] = (int32_t)base;
-                    for (int64_t lane = 0; lane < 32 && 32 * (int64_t)sl + lane < n; ++lane) {
-                        const int64_t k = sptr[sl] + 32 * j + lane;
-                        (*cd)[k] = (int16_t)((int64_t)scol[k] - lane - base);
-                    }
-                }
-            return true;
-        };
         sell(H.e_rp, H.e_col, hc.ne, &ptr, &w, &scol, &map);
         std::vector<double> sM = gather(map, H.M), sS = gather(map, H.S), sA = gather(map, A);
         std::vector<float> sA32(sA.begin(), sA.end());
@@ -1276,27 +764,12 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
             std::vector<double> pA = gather(map, val2);
             std::vector<float> pA32(pA.begin(), pA.end()), pdinv(ne);
             for (int64_t r = 0; r < ne; ++r) pdinv[r] = (float)Ad[(*perm)[r]];
-#ifdef FP_SMEM_REPORT
-            fprintf(stderr, "newmark solver order: %s, sectors %lld (edge order %lld), SELL slots %lld, nonzeros %lld\n",
-                    perm == &blocked ? "blocked" : "edge", (long long)F->sectors_e[1], (long long)F->sectors_e[0],
-                    (long long)scol.size(), (long long)H.e_col.size());
-#endif
             if (!d16.empty() && st == FP_OK) st = up(ctx, &F->se_d16, d16);
-            F->hptr[FP_SYS_NEWMARK] = ptr;
             F->hwidth[FP_SYS_NEWMARK] = w;
-            F->slots_total[FP_SYS_NEWMARK] = (int64_t)scol.size();
             if (st == FP_OK) st = up(ctx, &F->perm_e, *perm);
             if (st == FP_OK) st = up(ctx, &F->pe_ptr, ptr);
             if (st == FP_OK) st = up(ctx, &F->pe_w, w);
             if (st == FP_OK) st = up(ctx, &F->pe_col, scol);
-            {
-                std::vector<int32_t> cb;
-                std::vector<int16_t> cd;
-                if (FP_COL16 && columns16(scol, ptr, w, ne, &cb, &cd)) {
-                    if (st == FP_OK) st = up(ctx, &F->pe_cb, cb);
-                    if (st == FP_OK) st = up(ctx, &F->pe_cd, cd);
-                }
-            }
             if (st == FP_OK) st = up(ctx, &F->pe_A, pA);
             if (st == FP_OK) st = up(ctx, &F->pe_A32, pA32);
             if (st == FP_OK) st = up(ctx, &F->pe_dinv32, pdinv);
@@ -1309,21 +782,11 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
         {
             const std::vector<int16_t> d16 = offsets16(scol, ptr, w, hc.nn);
             if (!d16.empty() && st == FP_OK) st = up(ctx, &F->sn_d16, d16);
-            F->hptr[FP_SYS_GAUSS] = ptr;
             F->hwidth[FP_SYS_GAUSS] = w;
-            F->slots_total[FP_SYS_GAUSS] = (int64_t)scol.size();
         }
         if (st == FP_OK) st = up(ctx, &F->sn_ptr, ptr);
         if (st == FP_OK) st = up(ctx, &F->sn_w, w);
         if (st == FP_OK) st = up(ctx, &F->sn_col, scol);
-        {
-            std::vector<int32_t> cb;
-            std::vector<int16_t> cd;
-            if (FP_COL16 && columns16(scol, ptr, w, hc.nn, &cb, &cd)) {
-                if (st == FP_OK) st = up(ctx, &F->sn_cb, cb);
-                if (st == FP_OK) st = up(ctx, &F->sn_cd, cd);
-            }
-        }
         if (st == FP_OK) st = up(ctx, &F->sn_L, sL);
         if (st == FP_OK) st = up(ctx, &F->sn_L32, sL32);
     }
@@ -1345,10 +808,9 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
             if (d < best) best = d, *bs = b;
         }
         if (force > 0) *bs = force;
-        int per_sm = 0, per_sm2 = 0;
-        FP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(*bs, true), *bs, 0));
-        FP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, solver_kernel(*bs, false), *bs, 0));
-        per_sm = std::min(std::min(per_sm, per_sm2), kSolverPerSm);
+        int per_sm = 0;
+        FP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(*bs), *bs, 0));
+        per_sm = std::min(per_sm, kSolverPerSm);
         if (per_sm < 1) {
             ctx->err = "fem_pic_field_setup: the solver kernel cannot be co-resident";
             return FP_ECUDA;
@@ -1365,56 +827,19 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
 #endif
     if (st == FP_OK) st = pick(hc.ne, FP_SOLVER_BS_E, &F->bs_e, &F->grid_e);
     if (st == FP_OK) st = pick(hc.nn, FP_SOLVER_BS_N, &F->bs_n, &F->grid_n);
-    // Shared-memory residency of the FP32 operator in the mixed solver: the slots of a
-    // block's rows (its whole 32-row slices, as the kernel partitions them) must fit; the
-    // launch then stays co-resident with that much shared memory per block.
-    auto residency = [&](int sys, int64_t rows, int bs, int grid) -> fp_status {
-        F->sm_slots[sys] = 0;
-        const int16_t* d16 = sys == FP_SYS_NEWMARK ? F->se_d16 : F->sn_d16;
-        if (!d16 || grid < 1) return FP_OK;
-        const std::vector<int32_t>& ptr = F->hptr[sys];
-        const int64_t ns = (int64_t)ptr.size();
-        const int64_t chunk = ((rows + grid - 1) / grid + 31) & ~(int64_t)31;
-        int64_t most = 0;
-        for (int b = 0; b < grid; ++b) {
-            const int64_t r0 = std::min<int64_t>(rows, (int64_t)b * chunk), r1 = std::min<int64_t>(rows, r0 + chunk);
-            if (r0 >= r1) continue;
-            const int64_t s0 = r0 >> 5, s1 = (r1 + 31) >> 5;
-            const int64_t b1 = s1 < ns ? ptr[s1] : F->slots_total[sys];
-            most = std::max<int64_t>(most, b1 - ptr[s0]);
-        }
-        const int64_t slots = (most + 7) & ~(int64_t)7;        // int16 part starts 16-byte aligned
-        const size_t bytes = (size_t)slots * 6;
-        if (bytes > kSmemOperatorBytes) return FP_OK;
-        void* k = solver_kernel(bs, false);
-        // the attribute is per kernel, shared by every context: set it to the device's limit
-        // (less room for the kernel's static shared memory) so that no context lowers it below
-        // what another one launches with
-        int optin = 0;
-        FP_CUDA_TRY(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-        if (bytes + 4096 > (size_t)optin) return FP_OK;
-        FP_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 4096));
-        int per_sm = 0;
-        FP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, bs, bytes));
-        if ((int64_t)per_sm * ctx->sm_count < grid) return FP_OK;
-        F->sm_slots[sys] = (int)slots;
-        // room for the learned preconditioner's BF16 values beside them (8 bytes per slot)?
-        F->sm_learned[sys] = 0;
-        if ((size_t)slots * 8 <= kSmemOperatorBytes + 24 * 1024 && (size_t)slots * 8 + 4096 <= (size_t)optin) {
-            int per_sm8 = 0;
-            FP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm8, k, bs, (size_t)slots * 8));
-            F->sm_learned[sys] = (int64_t)per_sm8 * ctx->sm_count >= grid ? 1 : 0;
-        }
-        return FP_OK;
-    };
-#ifndef FP_SMEM_OPERATOR
-#define FP_SMEM_OPERATOR 1
-#endif
-    if (FP_SMEM_OPERATOR && st == FP_OK) st = residency(FP_SYS_NEWMARK, hc.ne, F->bs_e, F->grid_e);
-    if (FP_SMEM_OPERATOR && st == FP_OK) st = residency(FP_SYS_GAUSS, hc.nn, F->bs_n, F->grid_n);
+    // The mixed solver: on chip where a block's share of the operator fits in shared memory
+    // (pcg_resident.cu), streamed otherwise (pcg_stream.cu); both where the polynomial's two more
+    // vectors are what does not fit.
     for (int sys = 0; sys < 2 && st == FP_OK; ++sys)
         if (sys == FP_SYS_NEWMARK ? F->se_d16 : F->sn_d16)
             st = resident_setup(ctx, sys == FP_SYS_NEWMARK ? hc.ne : hc.nn, F->hwidth[sys], &F->res[sys]);
+    for (int sys = 0; sys < 2 && st == FP_OK; ++sys) {
+        if (F->res[sys].on && F->res[sys].smem_poly) continue;
+        const bool nm = sys == FP_SYS_NEWMARK;
+        const int wmax = F->hwidth[sys].empty() ? 0 : *std::max_element(F->hwidth[sys].begin(), F->hwidth[sys].end());
+        st = stream_setup(ctx, nm ? Sell{F->pe_ptr, F->pe_w, F->pe_col} : Sell{F->sn_ptr, F->sn_w, F->sn_col},
+                          nm ? F->pe_A : F->sn_L, nm ? F->pe_A32 : F->sn_L32, nm ? hc.ne : hc.nn, wmax, &F->stream[sys]);
+    }
     if (st == FP_OK) {
         FP_CUDA_TRY(ctx, cudaMalloc(&F->sync, grid_sync_bytes(ctx->sm_count)));
         FP_CUDA_TRY(ctx, cudaMemset(F->sync, 0, grid_sync_bytes(ctx->sm_count)));

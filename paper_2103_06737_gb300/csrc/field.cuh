@@ -5,16 +5,6 @@
 
 #include "internal.cuh"
 
-// FP_COL16=1: the mixed solver's streamed FP32 operators read their columns as 16-bit offsets
-// from a per-slice-position base (Sell::cb, Sell::cd) where every offset fits, a quarter fewer
-// operator bytes per product.  Measured on the 96^3 mesh (both operators streamed), Jacobi-CG
-// per solve: Newmark 17.8 -> 18.1 ms and Gauss-law 6.3 -> 6.8 ms in the bench; with the L2
-// prefetch of the operator, field-only, Newmark 19.5 -> 19.6 ms and Gauss-law 3.7 -> 4.2 ms.
-// The extra base load per entry costs more than the bytes it saves; off by default.
-#ifndef FP_COL16
-#define FP_COL16 0
-#endif
-
 namespace fempic {
 
 struct HostFields {
@@ -45,6 +35,19 @@ struct ResidentPlan {
     int32_t* pp = nullptr;      // device: slot pairs before each slice
 };
 
+// packed copies of one system's operator for the streamed mixed solver (pcg_stream.cu)
+struct StreamPlan {
+    bool on = false;
+    int64_t n = 0;
+    int ns = 0, nt = 0, nseg = 1, seg = 0, tpb = 0, grid = 0, ring = 0;   // slices, tiles, records per slice, their slots, tiles per block
+    void* where = nullptr;                // device: places of the learned correction's records
+    std::vector<uint32_t> width;          // per record: slots, and whether its columns are 32-bit
+    unsigned char* rec[3] = {nullptr, nullptr, nullptr};   // FP32, learned correction, FP64
+    uint2* meta[3] = {nullptr, nullptr, nullptr};
+    int stage[3] = {0, 0, 0};
+    size_t bytes[3] = {0, 0, 0};
+};
+
 struct FieldDev {
     double dt = 0, eps = 0, mu = 0;
     int bc = FP_BC_PEC;             // field boundary condition
@@ -71,27 +74,19 @@ struct FieldDev {
     float *r32 = nullptr, *z32 = nullptr, *p32 = nullptr, *q32 = nullptr, *c32 = nullptr;
     float *s32 = nullptr, *d32[2] = {nullptr, nullptr};  // Chebyshev preconditioner scratch
     double lmax[2] = {2.0, 2.0};    // estimated largest eigenvalue of D^-1 A, Newmark and Gauss systems
-    // FP32 operators held in shared memory by the mixed solver (per system): column offsets
-    // col - row as int16 in the SELL layout, and the slots per block (0: not held)
+    // column offsets col - row as int16 in the SELL layout, for the on-chip solver (null when some
+    // offset does not fit)
     int16_t *se_d16 = nullptr, *sn_d16 = nullptr;
-    // the 16-bit column encoding of the mixed solver's streamed operators (Sell::cb, Sell::cd):
-    // Newmark in the solver's row order, Gauss law (null when some offset does not fit)
-    int32_t *pe_cb = nullptr, *sn_cb = nullptr;
-    int16_t *pe_cd = nullptr, *sn_cd = nullptr;
     // The mixed solver's copy of the Newmark operator in its own row order: solver row r is
     // edge perm_e[r] (rows and columns renumbered alike).  Right-hand side and guess are
     // gathered into pb / px before each solve and the solution scattered back after it.
-    // se_d16 and hptr / slots_total of the Newmark system describe this copy.
+    // se_d16 and hwidth of the Newmark system describe this copy.
     int32_t *pe_ptr = nullptr, *pe_w = nullptr, *pe_col = nullptr, *perm_e = nullptr;
     double* pe_A = nullptr;
     float *pe_A32 = nullptr, *pe_dinv32 = nullptr;
     double *pb = nullptr, *px = nullptr;
     int64_t sectors_e[2] = {0, 0};  // gathered 32-byte sectors per product: edge order, solver order
-    int64_t slots_total[2] = {0, 0};
-    int sm_slots[2] = {0, 0};
-    int sm_learned[2] = {0, 0};     // the learned preconditioner's values fit in shared memory too
-    std::vector<int32_t> hptr[2];   // host copies of the SELL slice starts (Newmark, Gauss)
-    std::vector<int32_t> hwidth[2]; // and widths
+    std::vector<int32_t> hwidth[2];  // host copies of the SELL slice widths (Newmark, Gauss)
     double* red = nullptr;          // reduction partials
     double* out = nullptr;          // [8] solver outputs (iterations, rr, bb) of the last two solves
     int grid = 0;                   // co-resident blocks (cooperative launch limit)
@@ -99,7 +94,8 @@ struct FieldDev {
     int bs_e = 256, bs_n = 256;     // and their block sizes
     int last_fp64[2] = {0, 0};      // solver used by the last solve in each info slot
     ResidentPlan res[2];            // on-chip solver, Newmark and Gauss systems
-    void* sync = nullptr;           // words of the on-chip solver's grid exchanges (grid_sync.cuh)
+    StreamPlan stream[2];           // streamed solver, Newmark and Gauss systems
+    void* sync = nullptr;           // words of the mixed solvers' grid exchanges (grid_sync.cuh)
     LearnedDev* learned[2] = {nullptr, nullptr};  // per system (Newmark, Gauss)
     int learned_sys = FP_SYS_NEWMARK;              // system the fem_pic_learned_* calls address
     bool learned_used[2] = {false, false};         // the last solve in each info slot used its network
@@ -111,10 +107,6 @@ struct Sell {
     const int32_t* ptr;   // [slices] start of each slice
     const int32_t* w;     // [slices] width (longest row) of each slice
     const int32_t* col;   // padded entries point at the row itself with value 0
-    // the same columns in 16 bits (null when not built): column = cb[ptr/32 + j] + lane + cd,
-    // one 32-bit base per slice position j (the 32 lanes' j-th entries), a 16-bit offset per entry
-    const int32_t* cb = nullptr;
-    const int16_t* cd = nullptr;
 };
 
 // row i of a SELL-32 matrix times x; the 32 lanes of a warp take the 32 rows of a slice.
@@ -163,43 +155,6 @@ __device__ __forceinline__ X sell_row(const Sell& S, const V* __restrict__ val, 
         for (int u = 0; u < kSellChunk; ++u) s += (X)a[u] * xv[u];
     }
     return s;
-}
-
-// sell_row with the 16-bit column encoding (S.cd, S.cb non-null): 2 bytes per entry and one
-// base per 32 entries instead of 4 bytes per entry; the base is one broadcast load per warp
-template <typename V, typename X>
-__device__ __forceinline__ X sell_row16(const Sell& S, const V* __restrict__ val, const X* __restrict__ x,
-                                        int64_t i) {
-    const int64_t sl = i >> 5;
-    const int32_t p0 = __ldg(S.ptr + sl);
-    const int16_t* dp = S.cd + p0 + (i & 31);
-    const int32_t* bp = S.cb + (p0 >> 5);
-    const V* vp = val + p0 + (i & 31);
-    const int w = __ldg(S.w + sl);
-    const int lane = (int)(i & 31);
-    X s = X(0);
-    for (int j0 = 0; j0 < w; j0 += kSellChunk) {
-        int c[kSellChunk];
-        V a[kSellChunk];
-        X xv[kSellChunk];
-#pragma unroll
-        for (int u = 0; u < kSellChunk; ++u)
-            c[u] = j0 + u < w ? ld_op(bp + j0 + u) + lane + (int)ld_op(dp + 32 * (j0 + u)) : -1;
-#pragma unroll
-        for (int u = 0; u < kSellChunk; ++u) a[u] = j0 + u < w ? ld_op(vp + 32 * (j0 + u)) : V(0);
-#pragma unroll
-        for (int u = 0; u < kSellChunk; ++u) xv[u] = c[u] >= 0 ? __ldcg(x + c[u]) : X(0);
-#pragma unroll
-        for (int u = 0; u < kSellChunk; ++u) s += (X)a[u] * xv[u];
-    }
-    return s;
-}
-
-// the FP32 products of the mixed solver: 16-bit columns where built
-template <typename V, typename X>
-__device__ __forceinline__ X sell_row_any(const Sell& S, const V* __restrict__ val, const X* __restrict__ x,
-                                          int64_t i) {
-    return S.cd ? sell_row16<V, X>(S, val, x, i) : sell_row<V, X>(S, val, x, i);
 }
 
 #endif

@@ -44,6 +44,7 @@ struct GridSyncShared {
     float part[2][3][33];        // per-warp partials, by the exchange's parity
     float tot[2][2];
     unsigned long long prev[2][2];   // what each word held after this block's last exchange on it
+    int fail;                    // set by a thread whose own wait ran out: the block does not arrive any more
     int state[2];                // bit 0: a wait ran out, bit 1: add the partials one by one
 };
 
@@ -67,6 +68,7 @@ struct GridSync {
         // nothing changes the words at rest before every block's first arrival
         if (!ONE && threadIdx.x < 4) s->prev[threadIdx.x >> 1][threadIdx.x & 1] =
             *reinterpret_cast<volatile unsigned long long*>(mem + 8 * threadIdx.x);
+        if (threadIdx.x == 0) s->fail = 0;
         __syncthreads();
     }
     // by one thread at the end of a launch whose waits all ended: the next launch starts here
@@ -133,7 +135,7 @@ struct GridSync {
         if (threadIdx.x == 0) {
             const unsigned long long q[1] = {1ull};
             unsigned long long d[1];
-            const bool ok = arrive_wait<1>(par, q, d);
+            const bool ok = !sh->fail && arrive_wait<1>(par, q, d);
             if (!ok) atomicOr(status, ST_TIMEOUT);
             sh->state[par] = ok ? 0 : 1;
         }
@@ -167,7 +169,7 @@ struct GridSync {
         if (ONE) return true;
         float* parts = reinterpret_cast<float*>(mem + 3 * kGridLine + (size_t)par * nb * 24);
         if (threadIdx.x == 0) {
-            unsigned long long q[NV], d[NV];
+            unsigned long long q[NV], d[NV] = {};
             int e[NV];
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
@@ -177,7 +179,7 @@ struct GridSync {
                 q[k] = (fits ? (unsigned long long)__float2ll_rn(x) << 16 : 256ull) + 1ull;
                 parts[k * nb + blockIdx.x] = v[k];             // for the sums added one by one
             }
-            const bool ok = arrive_wait<NV>(par, q, d);
+            const bool ok = !sh->fail && arrive_wait<NV>(par, q, d);
             bool exact = false;
 #pragma unroll
             for (int k = 0; k < NV; ++k) {

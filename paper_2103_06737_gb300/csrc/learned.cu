@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "field.cuh"
+#include "pcg.cuh"
 
 namespace fempic {
 
@@ -1144,7 +1145,8 @@ fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_c
         P2[kOffDh] = 0.f;
         FP_CUDA_TRY(ctx, cudaMemcpy(L->params, P2.data(), kNParams * sizeof(float), cudaMemcpyHostToDevice));
         const bool nm2 = sys == FP_SYS_NEWMARK;
-        L->pre_slots = F->slots_total[sys];
+        L->pre_slots = 0;
+        for (int32_t w : F->hwidth[sys]) L->pre_slots += 32 * (int64_t)w;
         if (st == FP_OK) st = up(&L->xin, xin);
         if (st == FP_OK) st = up(&L->tpos, tpos);
         if (st == FP_OK) st = alloc(ctx, &L->delta, (size_t)nnz);
@@ -1153,6 +1155,7 @@ fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_c
         if (st == FP_OK) st = alloc(ctx, &L->u, n);
         if (st == FP_OK) st = alloc(ctx, &L->g, n);
         if (st == FP_OK) st = alloc(ctx, &L->pre, (size_t)std::max<int64_t>(1, L->pre_slots));
+        if (st == FP_OK) st = stream_learned_room(ctx, &F->stream[sys]);
         (void)nm2;
         if (st != FP_OK) return st;
     }
@@ -1315,6 +1318,10 @@ fp_status fem_pic_learned_build(fem_pic_t* ctx, void* stream) {
         nm ? F->pe_ptr : F->sn_ptr, nm ? F->pe_w : F->sn_w, nm ? F->pe_col : F->sn_col, nm ? F->pe_A : F->sn_L,
         nm ? F->perm_e : nullptr, L->dis, L->h[kLayers], L->params, L->fixed, L->n, L->pre);
     FP_CUDA_TRY(ctx, cudaGetLastError());
+    st = stream_learned_pack(ctx, &F->stream[L->sys],
+                             nm ? Sell{F->pe_ptr, F->pe_w, F->pe_col} : Sell{F->sn_ptr, F->sn_w, F->sn_col},
+                             nm ? F->pe_A : F->sn_L, L->pre, s);
+    if (st != FP_OK) return st;
     L->built = 1;
     return FP_OK;
 }

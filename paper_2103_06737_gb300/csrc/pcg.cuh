@@ -1,10 +1,30 @@
-// Interface of the mixed-precision solvers to the field step (field.cu).
+// The mixed-precision solvers of the field step (field.cu): iterative refinement.  The residual
+// r = b - A x and its norm are FP64; each correction A c = r / |r| is solved approximately by PCG
+// on FP32 copies of A and of the vectors, with FP32 sums (until its own residual drops by
+// inner_tol, or by less when that already meets the outer tolerance), then x += |r| c in FP64.
+// A p is carried as q = A z + beta q: two grid sums per inner iteration.
+//
+// Preconditioners of the inner PCG: Jacobi; a learned correction, z = D^-1 r + Dl r with Dl on the
+// operator's pattern (a solve in which r.z is not positive goes on with Jacobi); or z = P(r), P
+// the Chebyshev polynomial of degree deg in B = D^-1 A applied to f = D^-1 r (three-term
+// recurrence on [theta - delta, theta + delta]):
+//   d_0 = f / theta, z = d_0, s = f;
+//   k = 1..deg-1:  s <- s - B d_{k-1},  d_k = rho_k rho_{k-1} d_{k-1} + (2 rho_k / delta) s,
+//                  z <- z + d_k,  rho_0 = delta / theta,  rho_k = 1 / (2 theta / delta - rho_{k-1}).
+// P is positive on (0, theta + delta] and beyond it up to 2 theta, so PCG with it stays a
+// symmetric positive definite method.  Each step's product needs the previous d of every block:
+// one grid barrier per step, d in two buffers.
+//
+// One cooperative launch per solve; every block takes the same decisions from the same grid sums.
 #pragma once
 
 #include "field.cuh"
 
 namespace fempic {
 
+// fraction of the outer threshold an inner solve aims for when that needs less than inner_tol
+// (the FP32 recurrence residual can differ slightly from the FP64 one)
+constexpr double kInnerMargin = 0.2;
 constexpr int kResMaxSlices = 96;   // slices of a block of the on-chip solver, at most
 
 #ifdef __CUDACC__
@@ -39,6 +59,41 @@ struct ResidentArgs {
 
 fp_status resident_solve(fem_pic* ctx, const ResidentPlan& P, ResidentArgs a, cudaStream_t s);
 
+struct StreamArgs {
+    const unsigned char* rec[3];   // packed operators: FP32, learned correction, FP64
+    const uint2* meta[3];          // per tile: offset in 16-byte units, bytes
+    int stage[3], nst[3];          // bytes of a place in the ring, places
+    int ns, nt, nseg, tpb;         // slices, tiles, records per slice, tiles per block
+    bool evict_first, learned, x_zero;
+    int64_t n;
+    const float* dinv32;
+    const int32_t* perm;    // row -> DOF (null: rows in DOF order)
+    const double* b;        // right-hand side, DOF order
+    double* x;              // start and solution, DOF order
+    double *pb, *px;        // both in row order (b and x themselves without a permutation)
+    double* ax;             // null, or A x for the final x in DOF order
+    const double* scale_vec;   // row order (no permutation with it)
+    double* r64;
+    float *r, *z, *p, *q, *c, *s, *d0, *d1;
+    void* sync;
+    int deg;
+    float theta, delta;
+    double tol, inner_tol;
+    int max_iter, max_outer;
+    double* out;
+    int32_t* status;
+    int* lflag;
+};
+
+// the streamed solver: packed copies of an operator (val: FP64, val32: FP32, both in SELL order),
+// room for a learned correction's records and their packing, and a solve
+fp_status stream_setup(fem_pic* ctx, const Sell& S, const double* val, const float* val32, int64_t n, int wmax,
+                       StreamPlan* P);
+fp_status stream_learned_room(fem_pic* ctx, StreamPlan* P);
+fp_status stream_learned_pack(fem_pic* ctx, StreamPlan* P, const Sell& S, const double* val, const __nv_bfloat16* pre,
+                              cudaStream_t s);
+fp_status stream_solve(fem_pic* ctx, const StreamPlan& P, StreamArgs a, cudaStream_t s);
+
 // sell_row without the evict-first hint: the FP64 operator of an on-chip solve is read once
 // per refinement and stays in L2 between them
 __device__ __forceinline__ double sell_row_cached(const Sell& S, const double* __restrict__ val, const double* x,
@@ -62,6 +117,8 @@ __device__ __forceinline__ double sell_row_cached(const Sell& S, const double* _
     return s;
 }
 #endif
+
+void stream_free(StreamPlan* P);
 
 // plan of an on-chip solve; P->on stays false where the system does not fit
 fp_status resident_setup(fem_pic* ctx, int64_t n, const std::vector<int32_t>& width, ResidentPlan* P);

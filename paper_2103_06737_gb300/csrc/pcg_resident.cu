@@ -1,8 +1,7 @@
 // Mixed-precision field solve with everything an iteration touches held on chip.
 //
-// Same method as k_pcg_mixed (field.cu): iterative refinement with an FP64 residual and FP32
-// inner PCG (Jacobi, Chebyshev or learned preconditioner), used where a block's share of the
-// FP32 operator and of the solver's vectors fits in its shared memory.  A solve of such a system
+// The method is pcg.cuh's, here for systems of which a block's share of the FP32 operator and of
+// the solver's vectors fits in its shared memory.  A solve of such a system
 // moves almost no memory; its time is the latency of each iteration's chain: products that wait
 // on gathered entries, and grid-wide sums.  So here
 //  - a lane owns the same rows through the whole solve and keeps their r, z, p, q, c and D^-1
@@ -17,7 +16,8 @@
 //    the row permutation, without separate gather and scatter launches.
 // Bound by latency: per Jacobi iteration two exchanges (1.5 us each on 152 blocks), one product
 // (about 1 us for one slice a warp, 4 us for two slices a warp of the edge system).  Measured on
-// the 32^3 mesh, per solve, against k_pcg_mixed with the same operator in shared memory: edge
+// the 32^3 mesh, per solve, against a kernel with the same operator in shared memory,
+// vectors in global memory and cooperative-groups barriers: edge
 // system 619 -> 420 us (46 Jacobi iterations) and 565 -> 385 us (17 of degree 3), node system
 // 573 -> 380 us (84 Jacobi) and 253 -> 180 us (7 of degree 8); 4^3 mesh (one block) 141 -> 75 us and
 // 52 -> 20 us.  Two or three rows a lane in registers instead of shared memory spilled at the 80
@@ -31,8 +31,6 @@
 
 namespace fempic {
 namespace {
-
-constexpr double kInnerMargin = 0.2;   // as in field.cu
 
 // the two signed 16-bit column offsets of a slot pair, kept in 32-bit registers throughout (a
 // build that let them live in 16-bit registers spilled those and read out of range)
@@ -159,7 +157,7 @@ struct Resident {
             }
             return true;
         }
-        // Chebyshev recurrence (see chebyshev_apply in field.cu)
+        // Chebyshev recurrence (pcg.cuh)
         float *sr = at(RV_S), *d = at(RV_D);
         const float sig = a.theta / a.delta;
         float rho = 1.f / sig;

@@ -1,7 +1,9 @@
-"""The on-chip mixed solver (operator and vectors in shared memory, sums on the grid's arrivals).
+"""The mixed solvers: on chip (operator and vectors in shared memory) and streamed, with sums on the
+grid's arrivals.
 
-Sizes at its edges: one block (at most 1024 rows) and just above it, a few blocks, every SM with
-several slices per warp, partial last slices; Jacobi, the Chebyshev polynomial and a learned
+Sizes at their edges: one block (at most 1024 rows) and just above it, a few blocks, every SM with
+several slices per warp, partial last slices, the first edge systems that no longer fit on chip
+(41, 44: streamed); Jacobi, the Chebyshev polynomial and a learned
 correction; both boundary conditions; a start that is not zero and a second solve right after.
 The FP64 residual of each solution is formed on the CPU with the library's own operators: it may
 exceed the tolerance by its own rounding only (10%).
@@ -27,9 +29,9 @@ def _built():
     build.build()
 
 
-@pytest.mark.parametrize("n", [2, 4, 5, 9, 10, 17, 23, 32])
+@pytest.mark.parametrize("n", [2, 4, 5, 9, 10, 17, 23, 32, 41, 44])
 @pytest.mark.parametrize("bc", [F.FP_BC_PEC, F.FP_BC_NEUMANN])
-def test_onchip_solves_reach_the_tolerance(n, bc):
+def test_mixed_solves_reach_the_tolerance(n, bc):
     m = I.cube_mesh(n, 1.0, 0.1, seed=1)
     lib = F.FemPic(m.xyz, m.tets, F.FP_FP32)
     F.fem_pic_field_setup(lib.h, 0.2 * I.gyro_period(0.1), bc=bc)
