@@ -207,15 +207,65 @@ __device__ __forceinline__ void warp_run_reduce(int key, Real v[NV], unsigned* h
     *end_out = end;
 }
 
+// Of the faces in cand (l^b_k < 0) the one crossed first: the smallest fraction l^a_k / (l^a_k -
+// l^b_k), 0 where l^a_k <= 0, the lowest face of equal ones.
+//
+// With several candidates the fractions are compared in FP32 first: both terms of l^a_k - l^b_k
+// are positive, so the FP32 fraction is within 4 roundings (5e-7) of the exact one, and two that
+// differ by more than 1e-5 of the larger are ordered as in FP64.  Only closer ones are compared in
+// FP64, by cross-multiplication.  (The comparison ran in FP64 for every warp that held one
+// such lane, a fifth of the FP64 issue slots of the walk, which GB300's FP64 pipe bounds.)
+__device__ __forceinline__ int first_exit(const double la[4], const double lb[4], unsigned cand) {
+    if ((cand & (cand - 1u)) == 0u) return __ffs(cand) - 1;
+    int kx = -1;
+    float best = 0.f, second = 3.0e38f;   // the smallest and the second smallest fraction
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((cand >> k) & 1u)) continue;
+        float f = 0.f;
+        if (pos_strict(la[k])) {
+            const float a = d2f(la[k]), b = d2f(lb[k]);
+            f = __fdividef(a, a - b);
+            f = f > 1e-30f ? f : 1e-30f;   // positive, whatever underflowed: never taken for the clamped 0
+        }
+        if (kx < 0 || f < best) {
+            second = kx < 0 ? second : best;
+            best = f;
+            kx = k;
+        } else if (f < second) {
+            second = f;
+        }
+    }
+    // a clamped 0 comes first, the lowest face of several; positive fractions need a gap
+    if (best == 0.f || (best > 1e-20f && second - best > 1e-5f * second)) return kx;
+    double bn = 0.0, bd = 1.0;
+    kx = -1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((cand >> k) & 1u)) continue;
+        double num = la[k], den = la[k] - lb[k];
+        if (!pos_strict(num) || !pos_strict(den)) {  // fraction clamps to 0
+            num = 0.0;
+            den = 1.0;
+        } else if (num > den) {                      // fraction clamps to 1
+            num = 1.0;
+            den = 1.0;
+        }
+        if (kx < 0 || num * bd < bn * den) {
+            kx = k;
+            bn = num;
+            bd = den;
+        }
+    }
+    return kx;
+}
+
 // ---------------------------------------------------------------- FP64 walk
 // Straight path from xa to xb, both relative to the origin of the start tet c.  Every
-// piece deposits its 6 edge values, the end point its 4 node charges.  When `agg` is
-// non-null and the path stays inside c, the 10 values are returned in agg instead of
-// being added (return true) so the caller can reduce them across the warp.
+// piece deposits its 6 edge values, the end point its 4 node charges.
 //
 // FP64 is spent only on the exit test: the end point's barycentrics in each tet, the
-// crossing fraction and the carried crossing barycentrics.  The smallest fraction is
-// found by cross-multiplication (one division per crossing).  The deposit products are
+// crossing fraction (one division per crossing) and the carried crossing barycentrics.  The deposit products are
 // in Real; the current point, needed only when the walk stops early, is tracked in
 // Real as well.
 //
@@ -223,10 +273,10 @@ __device__ __forceinline__ void warp_run_reduce(int key, Real v[NV], unsigned* h
 // end point's charge minus its start point's (the start's, where a particle is removed for a
 // non-finite push), instead of the end point's charge.
 template <typename Real, typename DG = Real, typename DQ = DG>
-__device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo, int c,
+__device__ void walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo, int c,
                           const double xa[3], const double xb[3], double qw, int max_cross,
                           DG* __restrict__ dG, DQ* __restrict__ Q, int32_t* __restrict__ status,
-                          Real* agg, int* end_cell, double end_off[3], bool cc = false) {
+                          int* end_cell, double end_off[3], bool cc = false) {
     Geo G;
     TetTopo Tc;
     double la[4], rel[3], os[3];
@@ -244,7 +294,7 @@ __device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restr
             bary(G, xa, la);
             deposit_charge<Real, DQ>(Tc, la, -qw, Q);
         }
-        return false;
+        return;
     }
     load_geo(geo, c, G);
     load_topo(topo, c, Tc);
@@ -266,46 +316,13 @@ __device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restr
 #pragma unroll
         for (int k = 0; k < 4; ++k) cand |= (k != entry && neg_strict(lb[k])) ? (1u << k) : 0u;
         int kx = -1;
-        double smin = 0.0;
-        if (cand != 0u && (cand & (cand - 1u)) == 0u) {
-            // one candidate (the common crossing): l^a_k > 0 > l^b_k gives s in [0,1)
-            kx = __ffs(cand) - 1;
-            const double ak = kx == 0 ? la[0] : (kx == 1 ? la[1] : (kx == 2 ? la[2] : la[3]));
-            const double bk = kx == 0 ? lb[0] : (kx == 1 ? lb[1] : (kx == 2 ? lb[2] : lb[3]));
-            smin = pos_strict(ak) ? ak / (ak - bk) : 0.0;
-        } else if (cand != 0u) {
-            // several: the smallest fraction by cross-multiplication, one division
-            double bn = 0.0, bd = 1.0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (!((cand >> k) & 1u)) continue;
-                double num = la[k], den = la[k] - lb[k];
-                if (!pos_strict(num) || !pos_strict(den)) {  // fraction clamps to 0
-                    num = 0.0;
-                    den = 1.0;
-                } else if (num > den) {                      // fraction clamps to 1
-                    num = 1.0;
-                    den = 1.0;
-                }
-                if (kx < 0 || num * bd < bn * den) {
-                    kx = k;
-                    bn = num;
-                    bd = den;
-                }
-            }
-            smin = bn / bd;
+        if (cand != 0u) {
+            kx = first_exit(la, lb, cand);
         }
         if (kx < 0) {
             *end_cell = t;
 #pragma unroll
             for (int i = 0; i < 3; ++i) end_off[i] = rel[i];
-            if (nc == 0 && agg) {
-                piece_values<Real>(la, lb, qw, agg);
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    agg[6 + k] = to_real<Real>(qw) * to_real<Real>(cc ? lb[k] - la[k] : lb[k]);
-                return true;
-            }
             deposit_piece<Real, DG>(Tc, la, lb, qw, dG);
             if (cc && nc == 0) {   // still in the start tet: the change of its nodes' charge
                 double lq[4];
@@ -315,7 +332,7 @@ __device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restr
             } else {
                 deposit_charge<Real, DQ>(Tc, lb, qw, Q);
             }
-            return false;
+            return;
         }
         if (nc == max_cross) {  // bound reached: stop at the last crossing point
             if (!cc || nc > 0) deposit_charge<Real, DQ>(Tc, la, qw, Q);   // (cc, no crossing: no change)
@@ -323,8 +340,12 @@ __device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restr
             *end_cell = t;
 #pragma unroll
             for (int i = 0; i < 3; ++i) end_off[i] = to_f64(ca[i]) + (os[i] - G.o[i]);
-            return false;
+            return;
         }
+        // the crossing fraction: l^a_k > 0 > l^b_k gives a value in [0,1), otherwise it clamps to 0
+        const double ak = kx == 0 ? la[0] : (kx == 1 ? la[1] : (kx == 2 ? la[2] : la[3]));
+        const double bk = kx == 0 ? lb[0] : (kx == 1 ? lb[1] : (kx == 2 ? lb[2] : lb[3]));
+        const double smin = pos_strict(ak) ? ak / (ak - bk) : 0.0;
         double lc[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) lc[k] = (k == kx) ? 0.0 : la[k] + smin * (lb[k] - la[k]);
@@ -339,7 +360,7 @@ __device__ bool walk_fp64(const TetGeo* __restrict__ geo, const TetTopo* __restr
             *end_cell = -1;
 #pragma unroll
             for (int i = 0; i < 3; ++i) end_off[i] = to_f64(ca[i]) + (os[i] - G.o[i]);
-            return false;
+            return;
         }
         TetTopo Tn;
         load_topo(topo, tn, Tn);
@@ -445,16 +466,78 @@ __device__ __forceinline__ void fields64(const double* __restrict__ rec, int c, 
 }
 
 // ---------------------------------------------------------------- FP64 mode
-template <typename Real>
-__global__ void __launch_bounds__(256) k_push_deposit(
-    const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo, const double* __restrict__ f64,
-    int32_t* __restrict__ cell, Real* __restrict__ off,
-    Real* __restrict__ vel, int64_t n, int32_t nt, double qmdt2, Real dt, double qw, int max_cross,
-    int aggregate, Real* __restrict__ dG, Real* __restrict__ Q, int32_t* __restrict__ status, int cc) {
+// One particle per lane: the mover's step, and where the end point's barycentrics say that the
+// particle stays in its tet, its deposit.  Bound by GB300's FP64 pipe (two operations per clock and
+// SM, whatever the lanes' mask), so two things keep its work down:
+//  - a particle that leaves its tet (a few percent) goes to a queue of its warp and is walked with
+//    31 others of its kind (walk_fp64), not while the rest of the warp waits;
+//  - the deposits of a run of particles in one tet are summed from shared memory, a lane per value
+//    and third of the warp: 11 additions a lane and particle round, where a segmented shuffle
+//    reduction of 10 values takes 10 per doubling of the run (45 at 10 particles per tet).  The
+//    weight q w is applied once per sum.
+// 2M electrons on the 32^3 mesh: 839 us with the walk and the shuffle reduction inline, 559 us now (FP64 pipe 85% busy).
+constexpr int kPush64Threads = 256;
+struct Push64Warp {
+    double val[10][33];
+    double qx[3][64];     // queued particles' end points
+    int64_t qp[64];       // and indexes
+    int id[10][33];       // edge and node ids of each lane's tet
+    int key[32];          // its tet, -1: nothing to add
+};
+
+// Boris (leapfrog)
+struct Boris64 {
+    const double* __restrict__ rec;
+    double* __restrict__ vel;
+    int64_t n;
+    double h, dt;
+    __device__ __forceinline__ void operator()(int64_t p, int c, const double x[3], double xb[3]) const {
+        double v[3] = {vel[p], vel[n + p], vel[2 * n + p]}, E[3], B[3];
+        fields64(rec, c, x, E, B);
+        boris<double>(v, E, B, h);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            vel[i * n + p] = v[i];
+            xb[i] = step_pos(x[i], dt, v[i]);
+        }
+    }
+};
+
+// walks the m (at most 32) last queued particles of the warp
+__device__ __forceinline__ void walk_queued64(const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo,
+                                              int32_t* __restrict__ cell, double* __restrict__ off, int64_t n,
+                                              double qw, int max_cross, double* __restrict__ dG,
+                                              double* __restrict__ Q, int32_t* __restrict__ status, bool cc,
+                                              const Push64Warp& W, int first, int m) {
+    const int lane = threadIdx.x & 31;
+    if (lane < m) {
+        const int k = first + lane;
+        const int64_t p = W.qp[k];
+        const double xb[3] = {W.qx[0][k], W.qx[1][k], W.qx[2][k]};
+        const double xa[3] = {off[p], off[n + p], off[2 * n + p]};
+        int end_cell;
+        double end_off[3];
+        walk_fp64<double>(geo, topo, cell[p], xa, xb, qw, max_cross, dG, Q, status, &end_cell, end_off, cc);
+        cell[p] = end_cell;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) off[i * n + p] = end_off[i];
+    }
+    __syncwarp();
+}
+
+template <class Move>
+__device__ __forceinline__ void push64(Push64Warp& W, const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo,
+                                       int32_t* __restrict__ cell, double* __restrict__ off, int64_t n, int32_t nt,
+                                       double qw, int max_cross, int aggregate, double* __restrict__ dG,
+                                       double* __restrict__ Q, int32_t* __restrict__ status, bool cc,
+                                       const Move& move) {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n;
-         base += stride) {
+    // this lane's value and part of the warp in the summation
+    const int sv = lane % 10, part = lane / 10, from = 11 * part, to = part < 2 ? from + 11 : 32;
+    double* const out = sv < 6 ? dG : Q;
+    int queued = 0;
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
         const int64_t p = base + lane;
         int c = p < n ? cell[p] : -1;
         if (c >= nt) {
@@ -462,46 +545,93 @@ __global__ void __launch_bounds__(256) k_push_deposit(
             c = -1;
         }
         int key = -1;
-        Real agg[10];
-#pragma unroll
-        for (int k = 0; k < 10; ++k) agg[k] = (Real)0;
-        TetTopo T;
+        bool leaves = false;
+        double xb[3] = {0.0, 0.0, 0.0};
         if (c >= 0) {
-            load_topo(topo, c, T);
-            Real x[3] = {off[p], off[n + p], off[2 * n + p]};
-            Real v[3] = {vel[p], vel[n + p], vel[2 * n + p]};
-            double xa[3] = {(double)x[0], (double)x[1], (double)x[2]};
-            Real E[3], B[3];
-            fields64(f64, c, xa, E, B);
-            boris<Real>(v, E, B, (Real)qmdt2);
-            vel[p] = v[0];
-            vel[n + p] = v[1];
-            vel[2 * n + p] = v[2];
-            double xb[3];
+            const double x[3] = {off[p], off[n + p], off[2 * n + p]};
+            move(p, c, x, xb);
+            bool finite = true;
 #pragma unroll
-            for (int i = 0; i < 3; ++i) xb[i] = (double)step_pos(x[i], dt, v[i]);
-            int end_cell;
-            double end_off[3];
-            if (walk_fp64<Real>(geo, topo, c, xa, xb, qw, max_cross, dG, Q, status, aggregate ? agg : nullptr,
-                                &end_cell, end_off, cc != 0))
+            for (int i = 0; i < 3; ++i) finite = finite && finite_bits(x[i]) && finite_bits(xb[i]);
+            Geo G;
+            load_geo(geo, c, G);
+            double la[4], lb[4], d[4];
+            bary(G, x, la);
+            bary(G, xb, lb);
+            leaves = !finite || neg_strict(lb[0]) || neg_strict(lb[1]) || neg_strict(lb[2]) || neg_strict(lb[3]);
+            if (!leaves) {
                 key = c;
-            cell[p] = end_cell;
-            off[p] = (Real)end_off[0];
-            off[n + p] = (Real)end_off[1];
-            off[2 * n + p] = (Real)end_off[2];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) d[k] = lb[k] - la[k];
+                const double a[10] = {la[0] * d[1] - la[1] * d[0], la[0] * d[2] - la[2] * d[0],
+                                      la[0] * d[3] - la[3] * d[0], la[1] * d[2] - la[2] * d[1],
+                                      la[1] * d[3] - la[3] * d[1], la[2] * d[3] - la[3] * d[2],
+                                      cc ? d[0] : lb[0], cc ? d[1] : lb[1], cc ? d[2] : lb[2], cc ? d[3] : lb[3]};
+                TetTopo T;
+                load_topo(topo, c, T);
+                if (aggregate) {
+#pragma unroll
+                    for (int k = 0; k < 10; ++k) {
+                        W.val[k][lane] = a[k];
+                        W.id[k][lane] = k < 6 ? T.edge[k] : T.node[k - 6];
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) atomicAdd(dG + T.edge[k], qw * a[k]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) atomicAdd(Q + T.node[k], qw * a[6 + k]);
+                }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) off[i * n + p] = xb[i];
+            }
         }
         if (aggregate) {
-            unsigned heads;
-            int end;
-            warp_run_reduce<Real, 10>(key, agg, &heads, &end);
-            if (((heads >> lane) & 1u) && key >= 0) {
+            W.key[lane] = key;
+            __syncwarp();
+            if (lane < 30) {
+                int run = -1, id = 0;
+                double s = 0.0;
+                for (int i = from; i < to; ++i) {
+                    const int k = W.key[i];
+                    if (k != run) {
+                        if (run >= 0) atomicAdd(out + id, qw * s);
+                        run = k;
+                        s = 0.0;
+                        if (k >= 0) id = W.id[sv][i];
+                    }
+                    if (k >= 0) s += W.val[sv][i];
+                }
+                if (run >= 0) atomicAdd(out + id, qw * s);
+            }
+            __syncwarp();
+        }
+        const unsigned lv = __ballot_sync(kFull, leaves);
+        if (lv) {
+            if (leaves) {
+                const int k = queued + __popc(lv & ((1u << lane) - 1u));
+                W.qp[k] = p;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) atomicAdd(dG + T.edge[k], agg[k]);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) atomicAdd(Q + T.node[k], agg[6 + k]);
+                for (int i = 0; i < 3; ++i) W.qx[i][k] = xb[i];
+            }
+            queued += __popc(lv);
+            __syncwarp();
+            if (queued >= 32) {
+                queued -= 32;
+                walk_queued64(geo, topo, cell, off, n, qw, max_cross, dG, Q, status, cc, W, queued, 32);
             }
         }
     }
+    if (queued > 0) walk_queued64(geo, topo, cell, off, n, qw, max_cross, dG, Q, status, cc, W, 0, queued);
+}
+
+__global__ void __launch_bounds__(kPush64Threads) k_push_deposit64(
+    const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo, const double* __restrict__ f64,
+    int32_t* __restrict__ cell, double* __restrict__ off, double* __restrict__ vel, int64_t n, int32_t nt, double h,
+    double dt, double qw, int max_cross, int aggregate, double* __restrict__ dG, double* __restrict__ Q,
+    int32_t* __restrict__ status, int cc) {
+    __shared__ Push64Warp W[kPush64Threads / 32];
+    const Boris64 move{f64, vel, n, h, dt};
+    push64(W[threadIdx.x >> 5], geo, topo, cell, off, n, nt, qw, max_cross, aggregate, dG, Q, status, cc != 0, move);
 }
 
 // ---------------------------------------------------------------- FP32 mode
@@ -1715,7 +1845,7 @@ __global__ void __launch_bounds__(128) k_walk32(const TetGeo* __restrict__ geo,
         }
         int end_cell;
         double end_off[3];
-        walk_fp64<float, DG, DQ>(geo, topo, c, xa, xb, qw, max_cross, dG, Q, status, nullptr, &end_cell, end_off,
+        walk_fp64<float, DG, DQ>(geo, topo, c, xa, xb, qw, max_cross, dG, Q, status, &end_cell, end_off,
                                  cc != 0);
         cell[p] = end_cell;
 #pragma unroll
@@ -1803,66 +1933,36 @@ __global__ void __launch_bounds__(128) k_walk_adams32(const TetHot* __restrict__
         }
         int end_cell;
         double end_off[3];
-        walk_fp64<float>(geo, topo, c, xa, xe, qw, max_cross, dG, Q, status, nullptr, &end_cell, end_off);
+        walk_fp64<float>(geo, topo, c, xa, xe, qw, max_cross, dG, Q, status, &end_cell, end_off);
         cell[p] = end_cell;
 #pragma unroll
         for (int k = 0; k < 3; ++k) off[k * n + p] = d2f(end_off[k]);
     }
 }
 
-// FP64 Adams step: FP64 gather (Whitney-1/2 on the tet), the Adams update and the FP64 walk
-// with warp-aggregated deposits of the particles that stay in their tet.
-__global__ void __launch_bounds__(256) k_push_adams64(
+// FP64 Adams step: FP64 gather (Whitney-1/2 on the tet) and the Adams update, then as the Boris push.
+struct Adams64 {
+    const double* __restrict__ rec;
+    double* __restrict__ vel;
+    const AdamsStep<double>& A;
+    __device__ __forceinline__ void operator()(int64_t p, int c, const double x[3], double xb[3]) const {
+        const int64_t n = A.n;
+        const double v[3] = {vel[p], vel[n + p], vel[2 * n + p]};
+        double E[3], B[3], a[3], v1[3], hx[3], ha[3];
+        adams_history<double>(A, p, hx, ha);
+        fields64(rec, c, x, E, B);
+        adams_update<double>(A, x, v, E, B, hx, ha, a, v1, xb);
+        adams_store<double>(A, vel, p, v, a, v1);
+    }
+};
+__global__ void __launch_bounds__(kPush64Threads) k_push_adams64(
     const TetGeo* __restrict__ geo, const TetTopo* __restrict__ topo, const double* __restrict__ f64,
     int32_t* __restrict__ cell, double* __restrict__ off,
     double* __restrict__ vel, AdamsStep<double> A, int32_t nt, double qw, int max_cross, int aggregate,
     double* __restrict__ dG, double* __restrict__ Q, int32_t* __restrict__ status) {
-    const int lane = threadIdx.x & 31;
-    const int64_t n = A.n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const int64_t p = base + lane;
-        int c = p < n ? cell[p] : -1;
-        if (c >= nt) {
-            atomicOr(status, ST_INVAL);
-            c = -1;
-        }
-        int key = -1;
-        double agg[10];
-#pragma unroll
-        for (int k = 0; k < 10; ++k) agg[k] = 0.0;
-        TetTopo T;
-        if (c >= 0) {
-            load_topo(topo, c, T);
-            double x[3] = {off[p], off[n + p], off[2 * n + p]};
-            double v[3] = {vel[p], vel[n + p], vel[2 * n + p]};
-            double E[3], B[3], a[3], v1[3], xb[3], hx[3], ha[3];
-            adams_history<double>(A, p, hx, ha);
-            fields64(f64, c, x, E, B);
-            adams_update<double>(A, x, v, E, B, hx, ha, a, v1, xb);
-            adams_store<double>(A, vel, p, v, a, v1);
-            int end_cell;
-            double end_off[3];
-            if (walk_fp64<double>(geo, topo, c, x, xb, qw, max_cross, dG, Q, status, aggregate ? agg : nullptr,
-                                  &end_cell, end_off))
-                key = c;
-            cell[p] = end_cell;
-            off[p] = end_off[0];
-            off[n + p] = end_off[1];
-            off[2 * n + p] = end_off[2];
-        }
-        if (aggregate) {
-            unsigned heads;
-            int end;
-            warp_run_reduce<double, 10>(key, agg, &heads, &end);
-            if (((heads >> lane) & 1u) && key >= 0) {
-#pragma unroll
-                for (int k = 0; k < 6; ++k) atomicAdd(dG + T.edge[k], agg[k]);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) atomicAdd(Q + T.node[k], agg[6 + k]);
-            }
-        }
-    }
+    __shared__ Push64Warp W[kPush64Threads / 32];
+    const Adams64 move{f64, vel, A};
+    push64(W[threadIdx.x >> 5], geo, topo, cell, off, A.n, nt, qw, max_cross, aggregate, dG, Q, status, false, move);
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier that nothing arrives at,
@@ -2159,7 +2259,7 @@ fp_status launch_push_deposit(fem_pic* ctx, const double* e, const double* b, co
                                                                                ctx->hc.nt, ctx->d_field64);
         }
         PhaseTimer pt(ctx, PH_PUSH64, s);
-        k_push_deposit<double><<<grid, 256, 0, s>>>(ctx->d_geo, ctx->d_topo, ctx->d_field64, p->cell,
+        k_push_deposit64<<<grid, kPush64Threads, 0, s>>>(ctx->d_geo, ctx->d_topo, ctx->d_field64, p->cell,
                                                     (double*)p->off, (double*)p->vel, p->n, nt, qmdt2, dt,
                                                     qw, max_cross, agg, (double*)dG, (double*)Q,
                                                     ctx->d_status, cc);
@@ -2262,7 +2362,7 @@ fp_status launch_push_adams(fem_pic* ctx, const double* e, const double* b, cons
                                                                                ctx->hc.nt, ctx->d_field64);
         }
         PhaseTimer pt(ctx, PH_ADAMS, s);
-        k_push_adams64<<<grid_for(p->n, ctx->sm_count), 256, 0, s>>>(ctx->d_geo, ctx->d_topo, ctx->d_field64,
+        k_push_adams64<<<grid_for(p->n, ctx->sm_count), kPush64Threads, 0, s>>>(ctx->d_geo, ctx->d_topo, ctx->d_field64,
                                                                       p->cell, (double*)p->off, (double*)p->vel, A,
                                                                       nt, qw, max_cross, agg, (double*)dG,
                                                                       (double*)Q, ctx->d_status);
