@@ -230,7 +230,7 @@ void fem_pic_destroy(fem_pic_t* ctx) {
     void* ptrs[] = {ctx->d_geo,     ctx->d_topo,    ctx->d_xyz,     ctx->d_edges,
                     ctx->d_faces,   ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn,
                     ctx->d_orient,  ctx->d_status,  ctx->d_sort_count, ctx->d_sort_block,
-                    ctx->d_sort_rank, ctx->d_hot, ctx->d_field64, ctx->d_slow_idx, ctx->d_slow_count,
+                    ctx->d_sort_rank, ctx->d_sort_rec, ctx->d_hot, ctx->d_field64, ctx->d_slow_idx, ctx->d_slow_count,
                     ctx->d_node_wall, ctx->d_tet_faces};
     for (void* p : ptrs)
         if (p) cudaFree(p);

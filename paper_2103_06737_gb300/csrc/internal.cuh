@@ -141,6 +141,7 @@ struct fem_pic {
     int32_t* d_sort_count = nullptr;  // [nt + 2]
     int32_t* d_sort_block = nullptr;  // block sums
     int32_t* d_sort_rank = nullptr;   // [cap]
+    void* d_sort_rec = nullptr;       // [cap] records of eight reals, or null
     int64_t sort_cap = 0;
     std::string err;
 };
