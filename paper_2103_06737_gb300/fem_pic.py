@@ -74,6 +74,8 @@ def library_path() -> str:
 def lib():
     """Load libfempic.so (built in-tree by build.py).  Raises if it is not there."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -158,8 +160,14 @@ def _check(st: int, h=None):
         raise FemPicError(st, _err(h))
 
 
+# the current stream's handle without a torch.cuda.Stream object around it, where torch has the call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, torch.cuda.Stream):
         return ctypes.c_void_p(stream.cuda_stream)
@@ -179,6 +187,9 @@ def _ptr(t):
 
 
 def _need(t, dtype, numel=None, cuda=True, name="tensor"):
+    if (isinstance(t, torch.Tensor) and t.dtype == dtype and (t.is_cuda or not cuda)
+            and (numel is None or t.numel() == numel) and t.is_contiguous()):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
@@ -251,11 +262,21 @@ def fem_pic_last_error(h) -> str:
     return _err(h)
 
 
+_Sizes = ctypes.c_int64 * 5
+
+
+def _sizes(h):
+    """(N_n, N_e, N_f, N_t, precision)"""
+    s = _Sizes()
+    st = lib().fem_pic_sizes(h, ctypes.addressof(s))
+    if st != FP_OK:
+        _check(st, h)
+    return s
+
+
 def fem_pic_sizes(h) -> dict:
-    s = np.zeros(5, dtype=np.int64)
-    _check(lib().fem_pic_sizes(h, _ptr(s)), h)
-    return dict(n_nodes=int(s[0]), n_edges=int(s[1]), n_faces=int(s[2]), n_tets=int(s[3]),
-                precision=int(s[4]))
+    s = _sizes(h)
+    return dict(n_nodes=s[0], n_edges=s[1], n_faces=s[2], n_tets=s[3], precision=s[4])
 
 
 def fem_pic_incidence(h, which: int):
@@ -290,7 +311,7 @@ def fem_pic_project_uniform(h, E0, B0, e=None, b=None, stream=None):
 
 
 def _real(h):
-    return torch.float32 if fem_pic_sizes(h)["precision"] == FP_FP32 else torch.float64
+    return torch.float32 if _sizes(h)[4] == FP_FP32 else torch.float64
 
 
 def _dep(h):
@@ -337,61 +358,71 @@ def fem_pic_particles_to_global(h, cell, off, X, stream=None):
     _check(lib().fem_pic_particles_to_global(h, n, _ptr(cell), _ptr(off), _ptr(X), _stream(stream)), h)
 
 
-def _check_species(h, sp: Species):
+def _check_species(real, sp: Species):
     n = sp.n
     _need(sp.cell, torch.int32, n, name="cell")
-    _need(sp.off, _real(h), 3 * n, name="off")
-    _need(sp.vel, _real(h), 3 * n, name="vel")
+    _need(sp.off, real, 3 * n, name="off")
+    _need(sp.vel, real, 3 * n, name="vel")
 
 
 def fem_pic_push_deposit(h, e, b, sp: Species, dt: float, dG, Q, max_cross: int = 64, flags: int = 0,
                          stream=None):
-    sz = fem_pic_sizes(h)
-    _check_species(h, sp)
-    _need(e, torch.float64, sz["n_edges"], name="e")
-    _need(b, torch.float64, sz["n_faces"], name="b")
-    _need(dG, _dep(h), sz["n_edges"], name="dG")
-    _need(Q, _chg(h), sz["n_nodes"], name="Q")
+    sz = _sizes(h)
+    _check_species(torch.float32 if sz[4] == FP_FP32 else torch.float64, sp)
+    _need(e, torch.float64, sz[1], name="e")
+    _need(b, torch.float64, sz[2], name="b")
+    _need(dG, _dep(h), sz[1], name="dG")
+    _need(Q, _chg(h), sz[0], name="Q")
     p = sp.abi()
-    _check(lib().fem_pic_push_deposit(h, _ptr(e), _ptr(b), ctypes.byref(p), float(dt), int(max_cross),
-                                      _ptr(dG), _ptr(Q), int(flags), _stream(stream)), h)
+    st = lib().fem_pic_push_deposit(h, e.data_ptr(), b.data_ptr(), ctypes.byref(p), float(dt), int(max_cross),
+                                    dG.data_ptr(), Q.data_ptr(), int(flags), _stream(stream))
+    if st != FP_OK:
+        _check(st, h)
 
 
 def fem_pic_push_deposit_adams(h, e, b, sp: Species, hist, step: int, dt: float, dG, Q, max_cross: int = 64,
                                flags: int = 0, stream=None):
     """Adams-Bashforth particle step; hist is the 18*n planar derivative history (see the header)."""
-    sz = fem_pic_sizes(h)
-    R = _real(h)
-    _check_species(h, sp)
+    sz = _sizes(h)
+    R = torch.float32 if sz[4] == FP_FP32 else torch.float64
+    _check_species(R, sp)
     _need(hist, R, 18 * sp.n, name="hist")
-    _need(e, torch.float64, sz["n_edges"], name="e")
-    _need(b, torch.float64, sz["n_faces"], name="b")
-    _need(dG, R, sz["n_edges"], name="dG")
-    _need(Q, R, sz["n_nodes"], name="Q")
+    _need(e, torch.float64, sz[1], name="e")
+    _need(b, torch.float64, sz[2], name="b")
+    _need(dG, R, sz[1], name="dG")
+    _need(Q, R, sz[0], name="Q")
     p = sp.abi()
-    _check(lib().fem_pic_push_deposit_adams(h, _ptr(e), _ptr(b), ctypes.byref(p), _ptr(hist), int(step),
-                                            float(dt), int(max_cross), _ptr(dG), _ptr(Q), int(flags),
-                                            _stream(stream)), h)
+    st = lib().fem_pic_push_deposit_adams(h, e.data_ptr(), b.data_ptr(), ctypes.byref(p), hist.data_ptr(), int(step),
+                                          float(dt), int(max_cross), dG.data_ptr(), Q.data_ptr(), int(flags),
+                                          _stream(stream))
+    if st != FP_OK:
+        _check(st, h)
 
 
 def fem_pic_deposit_charge(h, sp: Species, Q, flags: int = 0, stream=None):
-    _check_species(h, sp)
-    _need(Q, _chg(h), fem_pic_sizes(h)["n_nodes"], name="Q")
+    sz = _sizes(h)
+    _check_species(torch.float32 if sz[4] == FP_FP32 else torch.float64, sp)
+    _need(Q, _chg(h), sz[0], name="Q")
     p = sp.abi()
-    _check(lib().fem_pic_deposit_charge(h, ctypes.byref(p), _ptr(Q), int(flags), _stream(stream)), h)
+    st = lib().fem_pic_deposit_charge(h, ctypes.byref(p), Q.data_ptr(), int(flags), _stream(stream))
+    if st != FP_OK:
+        _check(st, h)
 
 
 def fem_pic_sort(h, src: Species, dst: Species, stream=None):
-    _check_species(h, src)
-    _check_species(h, dst)
+    R = _real(h)
+    _check_species(R, src)
+    _check_species(R, dst)
     a, b = src.abi(), dst.abi()
-    _check(lib().fem_pic_sort(h, ctypes.byref(a), ctypes.byref(b), _stream(stream)), h)
+    st = lib().fem_pic_sort(h, ctypes.byref(a), ctypes.byref(b), _stream(stream))
+    if st != FP_OK:
+        _check(st, h)
 
 
 def fem_pic_sort_columns(h, src: Species, dst: Species, cols_src, cols_dst, ncols: int, stream=None):
-    _check_species(h, src)
-    _check_species(h, dst)
     R = _real(h)
+    _check_species(R, src)
+    _check_species(R, dst)
     _need(cols_src, R, ncols * src.n, name="cols_src")
     _need(cols_dst, R, ncols * src.n, name="cols_dst")
     a, b = src.abi(), dst.abi()
@@ -450,9 +481,9 @@ def fem_pic_field_solve(h, system: int, rhs, x, tol: float = 1e-10, max_iter: in
 
 def fem_pic_field_step(h, E_prev, E_cur, E_next, b, dG_half, dG_prev, Q_new, tol: float = 1e-10,
                        max_iter: int = 10000, precond: int = FP_PC_JACOBI, info: bool = True, stream=None):
-    sz = fem_pic_sizes(h)
+    ne = _sizes(h)[1]
     for t, nm in ((E_prev, "E_prev"), (E_cur, "E_cur"), (E_next, "E_next")):
-        _need(t, torch.float64, sz["n_edges"], name=nm)
+        _need(t, torch.float64, ne, name=nm)
     inf = (SolveInfo * 2)() if info else None
     st = lib().fem_pic_field_step(h, _ptr(E_prev), _ptr(E_cur), _ptr(E_next), _ptr(b), _ptr(dG_half),
                                   _ptr(dG_prev), _ptr(Q_new), float(tol), int(max_iter), int(precond),
