@@ -234,14 +234,30 @@ __global__ void k_spmv(Sell Sl, const double* __restrict__ val, const double* __
         y[i] = sell_row<double, double>(Sl, val, x, i);
 }
 
-// g_n = (D0^T [*eps] E)_n + Q_n on free nodes (ME = [*eps] E), 0 on PEC nodes
+// g_n = (D0^T [*eps] E)_n + Q_n on free nodes (ME = [*eps] E), 0 on PEC nodes; and, where b is
+// given, the Faraday update of the same step, b <- b - dt D1 (E1 + E0)/2 on face (i<j<k): +(i,j)
+// +(j,k) -(i,k).  E1 is the Newmark solution before the projection: the projection subtracts a
+// gradient (zero on PEC edges, whose nodes it leaves alone), and D1 D0 = 0, so its curl is that of
+// the projected field.  One launch for both, and the projection then runs in place: a copy and a
+// launch less (the field step's kernels beside the solves: 4^3 mesh 36 -> 30 us, 32^3 75 -> 62 us).
 template <typename Real>
 __global__ void k_gauss_rhs(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
                             const int8_t* __restrict__ sgn, const uint8_t* __restrict__ fixed,
                             const double* __restrict__ ME, const Real* __restrict__ Q, int64_t nn,
-                            double* __restrict__ g, double* __restrict__ qd) {
+                            double* __restrict__ g, double* __restrict__ qd, const int32_t* __restrict__ fe,
+                            const double* __restrict__ E1, const double* __restrict__ E0, double half_dt, int64_t nf,
+                            double* __restrict__ b) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += stride) {
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, all = b ? nn + nf : nn;
+    for (int64_t i = first; i < all; i += stride) {
+        if (i >= nn) {
+            const int64_t f = i - nn;
+            const int ij = __ldg(fe + 3 * f), jk = __ldg(fe + 3 * f + 1), ik = __ldg(fe + 3 * f + 2);
+            const double c = (__ldg(E1 + ij) + __ldg(E0 + ij)) + (__ldg(E1 + jk) + __ldg(E0 + jk)) -
+                             (__ldg(E1 + ik) + __ldg(E0 + ik));
+            b[f] -= half_dt * c;
+            continue;
+        }
         if (fixed[i]) {
             g[i] = 0.0;
             qd[i] = 0.0;
@@ -254,23 +270,13 @@ __global__ void k_gauss_rhs(const int32_t* __restrict__ ptr, const int32_t* __re
     }
 }
 
-// E_e <- E_e - (d_j - d_i) on free edges: the Gauss-law projection E - D0 d
+// E_e <- EN_e - (d_j - d_i) on free edges, 0 on PEC edges: the Gauss-law projection E - D0 d (E may be EN)
 __global__ void k_project(const int32_t* __restrict__ edges, const uint8_t* __restrict__ fixed,
-                          const double* __restrict__ d, const double* __restrict__ EN, int64_t ne,
-                          double* __restrict__ E) {
+                          const double* __restrict__ d, const double* EN, int64_t ne, double* E) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += stride)
-        E[e] = fixed[e] ? 0.0 : EN[e] - (d[edges[2 * e + 1]] - d[edges[2 * e]]);
-}
-
-// b <- b - dt D1 (E1 + E0)/2, face (i<j<k): +(i,j) +(j,k) -(i,k)
-__global__ void k_faraday(const int32_t* __restrict__ fe, const double* __restrict__ E1,
-                          const double* __restrict__ E0, double half_dt, int64_t nf, double* __restrict__ b) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += stride) {
-        const int ij = fe[3 * f], jk = fe[3 * f + 1], ik = fe[3 * f + 2];
-        const double c = (E1[ij] + E0[ij]) + (E1[jk] + E0[jk]) - (E1[ik] + E0[ik]);
-        b[f] -= half_dt * c;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += stride) {
+        const int2 ij = __ldg(reinterpret_cast<const int2*>(edges) + e);
+        E[e] = fixed[e] ? 0.0 : EN[e] - (__ldg(d + ij.y) - __ldg(d + ij.x));
     }
 }
 
@@ -450,7 +456,7 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
                           int max_iter, cudaStream_t s) {
     FieldDev* F = ctx->field;
     const bool f32 = dG_f32(ctx), q32 = Q_f32(ctx);   // dG, Q are float arrays
-    const int ge = grid_of(ctx, F->ne), gn = grid_of(ctx, F->nn);
+    const int ge = grid_of(ctx, F->ne);
     {
         PhaseTimer pt(ctx, PH_SOLVE, s);
         // u = 2E^n - E^{n-1} goes straight into E_next: it is also the solver's starting guess
@@ -481,13 +487,16 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
         PhaseTimer pt(ctx, PH_SOLVE, s);
         if (F->last_fp64[0])
             k_spmv<<<ge, kBlock, 0, s>>>(Sell{F->se_ptr, F->se_w, F->se_col}, F->se_M, E_next, F->ne, F->tmp);
+        // and the Faraday update of b, from E^N
+        const int gf = grid_of(ctx, b ? F->nn + F->nf : F->nn);
         if (q32)
-            k_gauss_rhs<float><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn, F->node_fixed,
-                                                     F->tmp, (const float*)Q_new, F->nn, F->rhs, F->qd);
+            k_gauss_rhs<float><<<gf, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn, F->node_fixed,
+                                                     F->tmp, (const float*)Q_new, F->nn, F->rhs, F->qd, F->face_edges,
+                                                     E_next, E_cur, 0.5 * F->dt, F->nf, b);
         else
-            k_gauss_rhs<double><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn,
+            k_gauss_rhs<double><<<gf, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn,
                                                       F->node_fixed, F->tmp, (const double*)Q_new, F->nn, F->rhs,
-                                                      F->qd);
+                                                      F->qd, F->face_edges, E_next, E_cur, 0.5 * F->dt, F->nf, b);
         FP_CUDA_TRY(ctx, cudaGetLastError());
         fp_status sn = neumann_rhs(ctx, s);
         if (sn != FP_OK) return sn;
@@ -505,9 +514,7 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
         PhaseTimer pt(ctx, PH_SOLVE, s);
         st = neumann_gauge(ctx, s);
         if (st != FP_OK) return st;
-        FP_CUDA_TRY(ctx, cudaMemcpyAsync(F->tmp, E_next, F->ne * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        k_project<<<ge, kBlock, 0, s>>>(ctx->d_edges, F->edge_fixed, F->delta, F->tmp, F->ne, E_next);
-        if (b) k_faraday<<<grid_of(ctx, F->nf), kBlock, 0, s>>>(F->face_edges, E_next, E_cur, 0.5 * F->dt, F->nf, b);
+        k_project<<<ge, kBlock, 0, s>>>(ctx->d_edges, F->edge_fixed, F->delta, E_next, F->ne, E_next);
         FP_CUDA_TRY(ctx, cudaGetLastError());
     }
     return FP_OK;
@@ -1015,10 +1022,12 @@ fp_status fem_pic_field_initial(fem_pic_t* ctx, const void* Q, double* E, double
     FP_CUDA_TRY(ctx, cudaMemsetAsync(F->tmp, 0, F->ne * sizeof(double), s));
     if (f32)
         k_gauss_rhs<float><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn, F->node_fixed, F->tmp,
-                                                 (const float*)Q, F->nn, F->rhs, F->qd);
+                                                 (const float*)Q, F->nn, F->rhs, F->qd, nullptr, nullptr, nullptr,
+                                                 0.0, 0, nullptr);
     else
         k_gauss_rhs<double><<<gn, kBlock, 0, s>>>(ctx->d_n2e_ptr, ctx->d_n2e_col, ctx->d_n2e_sgn, F->node_fixed,
-                                                  F->tmp, (const double*)Q, F->nn, F->rhs, F->qd);
+                                                  F->tmp, (const double*)Q, F->nn, F->rhs, F->qd, nullptr, nullptr, nullptr,
+                                                  0.0, 0, nullptr);
     fp_status st = neumann_rhs(ctx, s);
     if (st == FP_OK)
         st = run_pcg(ctx, FP_SYS_GAUSS, F->rhs, F->delta, tol, F->qd, max_iter, 1, s, nullptr, true);
