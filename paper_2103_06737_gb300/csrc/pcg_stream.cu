@@ -17,11 +17,11 @@
 //    bytes per lane.
 // Measured per Jacobi iteration, against a kernel that read columns and values from global memory
 // with an L2 prefetch one step ahead: edge system of the 64^3 mesh (1.9M rows) 67 -> 51 us, of
-// 96^3 (6.3M rows) 235 -> 186 us (945 MB: 75% of a 6.8 TB/s copy), node system of 96^3 31 -> 25 us.
+// 96^3 (6.3M rows) 235 -> 189 us (945 MB: 74% of a 6.8 TB/s copy), node system of 96^3 31 -> 25 us.
 // With only the copies (no gather, no vectors) a 64^3 pass takes 36 us; the rest is the
 // instructions per entry and the gather's latency.  Tried and slower: a ring per warp with
 // its own copies (58 us), two slices per warp at once on 12 warps (67 us), 19 or 23 consumer warps
-// (spills, 58 us).
+// (spills, 58 us), chunks of 8 gathers (52 us).
 #include <algorithm>
 #include <cmath>
 
@@ -56,6 +56,26 @@ __host__ __device__ __forceinline__ uint32_t val_bytes(uint32_t w, int op) {
 }
 __host__ __device__ __forceinline__ uint32_t rec_bytes(uint32_t w, bool wide, int op) {
     return w == 0 ? 0u : base_bytes(w, wide) + col_bytes(w, wide) + val_bytes(w, op);
+}
+
+// rows that a pass reads once: past L1, whose room the gathered vector needs
+template <typename T>
+__device__ __forceinline__ T ld_row(const T* p) {
+    if constexpr (sizeof(T) == 4) {
+        float v;
+        asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        return v;
+    } else {
+        double v;
+        asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+        return v;
+    }
+}
+__device__ __forceinline__ float4 ld_row4(const float* p) {
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
 }
 
 __device__ __forceinline__ uint64_t evict_first_policy() {
@@ -282,9 +302,9 @@ struct DirectionRows {       // q = A z + beta q, p = z + beta p, and the deferr
     __device__ __forceinline__ Row load(int64_t i) const {
         Row r;
         r.z = a.z[i];
-        r.p = first ? 0.f : __ldcs(a.p + i);
-        r.q = first ? 0.f : __ldcs(a.q + i);
-        r.c = first || c_first ? 0.f : __ldcs(a.c + i);
+        r.p = first ? 0.f : ld_row(a.p + i);
+        r.q = first ? 0.f : ld_row(a.q + i);
+        r.c = first || c_first ? 0.f : ld_row(a.c + i);
         return r;
     }
     __device__ __forceinline__ void apply(int64_t i, const Row& r, float w) {
@@ -301,7 +321,7 @@ struct LearnedRows {         // z = D^-1 r + Dl r
     struct Row {
         float r, di;
     };
-    __device__ __forceinline__ Row load(int64_t i) const { return Row{a.r[i], __ldcs(a.dinv32 + i)}; }
+    __device__ __forceinline__ Row load(int64_t i) const { return Row{a.r[i], ld_row(a.dinv32 + i)}; }
     __device__ __forceinline__ void apply(int64_t i, const Row& r, float t) {
         const float zi = r.di * r.r + t;
         a.z[i] = zi;
@@ -318,7 +338,7 @@ struct ChebyshevRows {       // one step of the recurrence (pcg.cuh)
         float di, s, d, z, r;
     };
     __device__ __forceinline__ Row load(int64_t i) const {
-        return Row{__ldcs(a.dinv32 + i), __ldcs(a.s + i), dc[i], __ldcs(a.z + i), dn ? 0.f : __ldcs(a.r + i)};
+        return Row{ld_row(a.dinv32 + i), ld_row(a.s + i), dc[i], ld_row(a.z + i), dn ? 0.f : ld_row(a.r + i)};
     }
     __device__ __forceinline__ void apply(int64_t i, const Row& r, float t) {
         const float sn = r.s - r.di * t, dk = c1 * r.d + c2 * sn, zk = r.z + dk;
@@ -339,7 +359,7 @@ struct ResidualRows {        // r64 = b - A x
     struct Row {
         double b, s;
     };
-    __device__ __forceinline__ Row load(int64_t i) const { return Row{__ldcs(a.pb + i), ref && a.scale_vec ? __ldcs(a.scale_vec + i) : 0.0}; }
+    __device__ __forceinline__ Row load(int64_t i) const { return Row{ld_row(a.pb + i), ref && a.scale_vec ? ld_row(a.scale_vec + i) : 0.0}; }
     __device__ __forceinline__ void apply(int64_t i, const Row& r, double t) {
         const double ri = r.b - t;
         a.r64[i] = ri;
@@ -411,13 +431,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
                 const int64_t q = qa + k * qs;
                 di[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (q >= q1) continue;
-                if (!use_l) di[k] = __ldcs(reinterpret_cast<const float4*>(a.dinv32) + q);
+                if (!use_l) di[k] = ld_row4(a.dinv32 + 4 * q);
                 if (init) {
                     x0[k] = reinterpret_cast<const double2*>(a.r64)[2 * q];
                     x1[k] = reinterpret_cast<const double2*>(a.r64)[2 * q + 1];
                 } else {
-                    o[k] = __ldcs(reinterpret_cast<const float4*>(a.r) + q);
-                    y[k] = __ldcs(reinterpret_cast<const float4*>(a.q) + q);
+                    o[k] = ld_row4(a.r + 4 * q);
+                    y[k] = ld_row4(a.q + 4 * q);
                 }
             }
 #pragma unroll
