@@ -40,7 +40,7 @@ inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * b
 #ifdef __CUDACC__
 
 struct GridSyncShared {
-    double part64[3][33];
+    double part64[3][32];
     float part[2][3][33];        // per-warp partials, by the exchange's parity
     float tot[2][2];
     unsigned long long prev[2][2];   // what each word held after this block's last exchange on it
@@ -213,25 +213,37 @@ struct GridSync {
         return sh->state[par] != 1;
     }
 
-    // FP64 sums of three values (once per refinement), added in block order
-    __device__ __forceinline__ bool sum64(double (&v)[3]) {
+    // v[0..2] summed over the lanes of a warp: the totals in lanes 0, 8 and 16.  The values share the
+    // first two steps, six additions instead of fifteen: an FP64 instruction of a warp takes the
+    // SM's FP64 pipe 16 cycles, and every warp of a block issues these.
+    __device__ __forceinline__ double warp_sum3(const double (&v)[3]) const {
+        const bool h = lane & 16, q = lane & 8;
+        const double a = (h ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h ? v[0] : v[2], 16);
+        const double up = __shfl_xor_sync(0xffffffffu, v[1], 16), b = h ? 0.0 : v[1] + up;
+        double t = (q ? b : a) + __shfl_xor_sync(0xffffffffu, q ? a : b, 8);
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) sh->part64[k][wid] = v[k];
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        return t;
+    }
+
+    // FP64 sums of three values over the grid (once per refinement), added in block order, handed to
+    // post(v) in one thread of each block; what it writes to shared memory every thread sees
+    // after.  Scalar FP64 work belongs there: a square root or a quotient that every warp
+    // computes for itself keeps the FP64 pipe of the SM for microseconds.
+    template <class Post>
+    __device__ __forceinline__ bool sum64(double (&v)[3], Post post) {
+        const double t = warp_sum3(v);
+        if ((lane & 7) == 0 && lane < 24) sh->part64[lane >> 3][wid] = t;
         __syncthreads();
         double* parts = reinterpret_cast<double*>(mem + 3 * kGridLine + (size_t)(turn & 1u) * nb * 24);
         if (wid == 0) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                v[k] = lane < warps ? sh->part64[k][lane] : 0.0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-                if (!ONE && lane == 0) parts[k * nb + blockIdx.x] = v[k];
-            }
+            for (int k = 0; k < 3; ++k) v[k] = lane < warps ? sh->part64[k][lane] : 0.0;
+            const double b = warp_sum3(v);
+            if (ONE)
+                v[0] = b;
+            else if ((lane & 7) == 0 && lane < 24)
+                parts[(lane >> 3) * nb + blockIdx.x] = b;
         }
         if (!ONE && !barrier()) return false;
         if (wid == 0) {
@@ -240,19 +252,12 @@ struct GridSync {
                 for (int b = lane; b < nb; b += 32)
 #pragma unroll
                     for (int k = 0; k < 3; ++k) v[k] += __ldcg(parts + k * nb + b);
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+                v[0] = warp_sum3(v);
             }
-            if (lane == 0)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) sh->part64[k][32] = v[k];
+            const double all[3] = {v[0], __shfl_sync(0xffffffffu, v[0], 8), __shfl_sync(0xffffffffu, v[0], 16)};
+            if (lane == 0) post(all);
         }
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = sh->part64[k][32];
-        __syncthreads();   // part64 has one copy
         return true;
     }
 };

@@ -219,7 +219,7 @@ struct Resident {
     }
 
     // the whole solve; false when a wait ran out (in every thread of the block alike)
-    __device__ bool solve(int& total, int& outer, double& rr64, double& ref2, double& thr) {
+    __device__ bool solve(int& total, int& outer, Refinement& f) {
         const bool b0t0 = blockIdx.x == 0 && threadIdx.x == 0;
         bool use_l = a.dl16 != nullptr;   // every block takes the same decisions (grid sums)
         if (use_l && a.lflag && b0t0) *a.lflag = 0;
@@ -251,16 +251,12 @@ struct Resident {
                     }
                 }
             }
-            if (!g.sum64(v)) return false;
-            rr64 = v[0];
-            if (outer == 0) {
-                ref2 = a.scale_vec ? v[2] : v[1];
-                thr = a.tol * a.tol * ref2;
-            }
-            if (!(rr64 > thr) || total >= a.max_iter || outer >= a.max_outer) return true;
+            if (!g.sum64(v, [&](const double (&t)[3]) { f.set(t, outer == 0, a.scale_vec, a.tol, a.inner_tol); }))
+                return false;
+            if (f.stop || total >= a.max_iter || outer >= a.max_outer) return true;
             ++outer;
             // ---- inner FP32 PCG on A c = r / ||r||
-            const double rnorm = sqrt(rr64), rinv = 1.0 / rnorm;
+            const double rinv = f.rinv;
             for (int s = warp; s < nsl; s += W) {
                 const int i = 32 * s + lane, row = 32 * s0 + i;
                 if (row >= a.n) continue;
@@ -281,9 +277,7 @@ struct Resident {
             float rz = w[0], rr = w[1], pq = y[0];
             // by how much each sum changed last, for what to expect of the next
             float g_rz = 1.f, g_rr = 1.f, g_pq = 1.f;
-            const double need = kInnerMargin * sqrt(thr / rr64);
-            const float red = (float)(need > a.inner_tol ? need : a.inner_tol);
-            const float ithr = red * red * rr;
+            const float ithr = f.red * f.red * rr;
             for (;;) {
                 if (!(pq > 0.f) || total >= a.max_iter) break;
                 const float alpha = rz / pq;
@@ -307,6 +301,7 @@ struct Resident {
                 g_pq = y[0] / pq;
                 pq = y[0];
             }
+            const double rnorm = f.rnorm;
             for (int s = warp; s < nsl; s += W) {
                 const int i = 32 * s + lane, row = 32 * s0 + i;
                 if (row < a.n) px[row] += rnorm * f2d(c[i]);
@@ -321,6 +316,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ GridSyncShared shs;
     __shared__ int sp[kResMaxSlices + 1];
+    __shared__ Refinement f;
     GridSync<ONE> g;
     g.init(a.sync, &shs, a.status);
     Resident<THREADS, ONE> S{a, g};
@@ -334,8 +330,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
     S.vec = reinterpret_cast<float*>(dsm + (size_t)a.pairs_max * 32 * 12);
     S.xz = a.z, S.x0 = a.d0, S.x1 = a.d1;
     if (ONE) {
-        float* f = S.vec + (a.deg > 1 ? RV_COUNT : RV_JACOBI) * S.rows_pb;
-        S.xz = f, S.x0 = f + S.rows_pb, S.x1 = f + 2 * S.rows_pb;
+        float* v = S.vec + (a.deg > 1 ? RV_COUNT : RV_JACOBI) * S.rows_pb;
+        S.xz = v, S.x0 = v + S.rows_pb, S.x1 = v + 2 * S.rows_pb;
     }
     for (int s = threadIdx.x; s <= S.nsl; s += blockDim.x) sp[s] = __ldg(a.pp + S.s0 + s) - __ldg(a.pp + S.s0);
     __syncthreads();
@@ -361,8 +357,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
         }
     }
     int total = 0, outer = 0;
-    double rr64 = 0.0, ref2 = 0.0, thr = 0.0;
-    const bool done = S.solve(total, outer, rr64, ref2, thr);
+    const bool done = S.solve(total, outer, f);
     if (done) {
         for (int s = S.warp; s < S.nsl; s += S.W) {
             const int row = 32 * (S.s0 + s) + S.lane;
@@ -375,10 +370,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
     if (done && blockIdx.x == 0 && threadIdx.x == 0) {
         g.finish();
         a.out[0] = (double)total;
-        a.out[1] = rr64;
-        a.out[2] = ref2;
+        a.out[1] = f.rr;
+        a.out[2] = f.ref2;
         a.out[3] = (double)outer;
-        if (rr64 > thr) atomicOr(a.status, ST_NOCONV);
+        if (f.rr > f.thr) atomicOr(a.status, ST_NOCONV);
     }
 }
 

@@ -396,8 +396,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
     const int64_t q0 = r0 / 4 + threadIdx.x, q1 = r1 / 4, qs = blockDim.x;
     const int64_t rest = 4 * q1 + threadIdx.x;   // the last rows of a count that is no multiple of 4
     const bool b0t0 = blockIdx.x == 0 && threadIdx.x == 0;
+    __shared__ Refinement ref;
     int total = 0, outer = 0;
-    double rr64 = 0.0, ref2 = 0.0, thr = 0.0;
     bool use_l = a.learned;   // every block takes the same decisions (grid sums)
     if (use_l && a.lflag && b0t0) *a.lflag = 0;
     auto product_op = [&]() { return use_l ? OP_LEARNED : OP_F32; };   // the first product of an iteration
@@ -523,19 +523,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
                 v[0] = f.rr, v[1] = f.bb, v[2] = f.ss;
             }
             R.start(product_op());
-            if (!g.sum64(v)) return false;
-            rr64 = v[0];
-            if (outer == 0) {
-                ref2 = a.scale_vec ? v[2] : v[1];
-                thr = a.tol * a.tol * ref2;
-            }
-            if (!(rr64 > thr) || total >= a.max_iter || outer >= a.max_outer) return true;
+            if (!g.sum64(v, [&](const double (&t)[3]) { ref.set(t, outer == 0, a.scale_vec, a.tol, a.inner_tol); }))
+                return false;
+            if (ref.stop || total >= a.max_iter || outer >= a.max_outer) return true;
             ++outer;
             // ---- inner FP32 PCG on A c = r / ||r||
-            const double rnorm = sqrt(rr64);
-            rinv = 1.0 / rnorm;
-            const double need = kInnerMargin * sqrt(thr / rr64);
-            const float red = (float)(need > a.inner_tol ? need : a.inner_tol);
+            rinv = ref.rinv;
             float rz = 0.f, rr = 0.f, pq = 0.f, ithr = 0.f;
             float g_rz = 1.f, g_rr = 1.f, g_pq = 1.f;   // by how much each sum changed last
             // init: the first direction; c_first: c holds nothing yet; step: c += alpha p is still to
@@ -558,7 +551,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
                 }
                 DirectionRows f{a, init, c_first, init ? 0.f : w[0] / rz, alpha, 0.f};
                 rz = w[0], rr = w[1];
-                if (init) ithr = red * red * rr;
+                if (init) ithr = ref.red * ref.red * rr;
                 stream_pass<OP_F32>(R, a.z, f);
                 R.start(product_op());
                 float y[1] = {f.pq};
@@ -578,6 +571,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
             R.start(OP_F64);
             if (restart) continue;   // x is unchanged: the refinement starts again with Jacobi
             // x += ||r|| c, with the last step's alpha p
+            const double rnorm = ref.rnorm;
             if (!c_first || step)
                 for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
                     const float ci = c_first ? 0.f : a.c[i];
@@ -598,10 +592,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
     if (b0t0) {
         g.finish();
         a.out[0] = (double)total;
-        a.out[1] = rr64;
-        a.out[2] = ref2;
+        a.out[1] = ref.rr;
+        a.out[2] = ref.ref2;
         a.out[3] = (double)outer;
-        if (rr64 > thr) atomicOr(a.status, ST_NOCONV);
+        if (ref.rr > ref.thr) atomicOr(a.status, ST_NOCONV);
     }
 }
 
