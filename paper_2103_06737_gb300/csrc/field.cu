@@ -180,32 +180,32 @@ __global__ void __launch_bounds__(BS, BS >= 1024 ? 1 : kSolverPerSm) k_pcg(PcgAr
     }
 }
 
-// Newmark right-hand side and the extrapolated initial guess 2E^n - E^{n-1}, in two passes
-// so that the SELL pass does two FP64 multiply-adds per stored entry:
-//   u = 2E^n - E^{n-1} (also the guess), v = -dt^2 (E^n / 2 + E^{n-1} / 4)   (per row)
-//   rhs = [*eps] u + [*S] v - (dG^{n+1/2} - dG^{n-1/2})                      (SELL)
-__global__ void k_newmark_uv(const uint8_t* __restrict__ fixed, const double* __restrict__ En,
-                             const double* __restrict__ Em, double dt2, int64_t n, double* __restrict__ u,
-                             double* __restrict__ v) {
+// Newmark right-hand side, the extrapolated initial guess u = 2E^n - E^{n-1} and its residual.
+// With A = [*eps] + dt^2/4 [*S] the right-hand side
+//   [*eps] u - dt^2 [*S] (E^n / 2 + E^{n-1} / 4) - dG = A u - dt^2 [*S] E^n - dG,
+// dG = dG^{n+1/2} - dG^{n-1/2}: so r0 = b - A u = -dt^2 [*S] E^n - dG comes with it, and the solver
+// starts without an FP64 product of its own (field step on the 64^3 mesh 2423 -> 2383 us, 96^3
+// 18.0 -> 17.5 ms).
+// u is a pass of its own, so that the SELL pass does two FP64 multiply-adds per stored entry.
+__global__ void k_newmark_guess(const uint8_t* __restrict__ fixed, const double* __restrict__ En,
+                                const double* __restrict__ Em, int64_t n, double* __restrict__ u) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const double en = En[i], em = Em[i];
-        u[i] = fixed[i] ? 0.0 : 2.0 * en - em;
-        v[i] = -dt2 * (0.5 * en + 0.25 * em);
-    }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+        u[i] = fixed[i] ? 0.0 : 2.0 * En[i] - Em[i];
 }
 
 template <typename Real>
-__global__ void k_newmark_rhs(Sell Sl, const double* __restrict__ Mv, const double* __restrict__ Sv,
+__global__ void k_newmark_rhs(Sell Sl, const double* __restrict__ Av, const double* __restrict__ Sv,
                               const uint8_t* __restrict__ fixed, const double* __restrict__ u,
-                              const double* __restrict__ v, const Real* __restrict__ dGh,
-                              const Real* __restrict__ dGp, int64_t n, double* __restrict__ rhs) {
+                              const double* __restrict__ En, double dt2, const Real* __restrict__ dGh,
+                              const Real* __restrict__ dGp, int64_t n, double* __restrict__ rhs,
+                              double* __restrict__ r0) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const int64_t sl = i >> 5;
         const int64_t base = __ldg(Sl.ptr + sl) + (i & 31);
         const int w = __ldg(Sl.w + sl);
-        double s = 0.0;
+        double s = 0.0, t = 0.0;
         for (int j0 = 0; j0 < w; j0 += kSellChunk) {   // chunks of independent loads, as in sell_row
             int c[kSellChunk];
 #pragma unroll
@@ -214,16 +214,18 @@ __global__ void k_newmark_rhs(Sell Sl, const double* __restrict__ Mv, const doub
             for (int q = 0; q < kSellChunk; ++q) {
                 if (c[q] < 0) continue;
                 const int64_t k = base + 32 * (int64_t)(j0 + q);
-                s = fma(__ldg(Mv + k), u[c[q]], s);
-                s = fma(__ldg(Sv + k), v[c[q]], s);
+                s = fma(__ldg(Av + k), u[c[q]], s);
+                t = fma(__ldg(Sv + k), __ldg(En + c[q]), t);
             }
         }
         if (fixed[i]) {
-            rhs[i] = 0.0;
+            rhs[i] = r0[i] = 0.0;
             continue;
         }
         const double gh = dGh ? as_f64(dGh[i]) : 0.0, gp = dGp ? as_f64(dGp[i]) : 0.0;
-        rhs[i] = s - (gh - gp);
+        const double r = -dt2 * t - (gh - gp);
+        r0[i] = r;
+        rhs[i] = s + r;
     }
 }
 
@@ -308,7 +310,8 @@ fp_status up(fem_pic* ctx, T** d, const std::vector<T>& h) {
 // mixed solver ran (F->last_fp64[slot] == 0 afterwards); the FP64 solver leaves it alone.
 // x_zero: the start is zero whatever x holds.
 fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double tol, const double* scale_vec,
-                  int max_iter, int slot, cudaStream_t s, double* ax = nullptr, bool x_zero = false) {
+                  int max_iter, int slot, cudaStream_t s, double* ax = nullptr, bool x_zero = false,
+                  const double* r0 = nullptr) {
     FieldDev* F = ctx->field;
     int use64 = ctx->solver_fp64;
     if (ctx->solver_sys[system] >= 0) use64 = ctx->solver_sys[system] == FP_PC_JACOBI_FP64;
@@ -335,7 +338,7 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
             a.dinv32 = nm ? F->pe_dinv32 : F->Ldinv32, a.dl16 = dl16, a.perm = perm;
             a.n = nm ? F->ne : F->nn, a.ns = (int)((a.n + 31) / 32);
             a.b = rhs, a.x = x, a.px = perm ? F->px : x, a.ax = ax, a.x_zero = x_zero, a.scale_vec = scale_vec;
-            a.r64 = F->q, a.z = F->z32, a.d0 = F->d32[0], a.d1 = F->d32[1], a.sync = F->sync;
+            a.r0 = x_zero ? rhs : r0, a.r64 = F->q, a.z = F->z32, a.d0 = F->d32[0], a.d1 = F->d32[1], a.sync = F->sync;
             a.deg = deg, a.theta = theta, a.delta = delta, a.tol = tol, a.inner_tol = ctx->inner_tol;
             a.max_iter = max_iter, a.max_outer = max_outer, a.out = F->out + 4 * slot, a.status = ctx->d_status;
             a.lflag = lflag;
@@ -345,7 +348,7 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
         a.learned = dl16 != nullptr, a.x_zero = x_zero;
         a.dinv32 = nm ? F->pe_dinv32 : F->Ldinv32, a.perm = perm;
         a.b = rhs, a.x = x, a.pb = perm ? F->pb : const_cast<double*>(rhs), a.px = perm ? F->px : x, a.ax = ax;
-        a.scale_vec = scale_vec, a.r64 = F->q;
+        a.scale_vec = scale_vec, a.r0 = x_zero ? rhs : r0, a.r64 = F->q;
         a.r = F->r32, a.z = F->z32, a.p = F->p32, a.q = F->q32, a.c = F->c32, a.s = F->s32;
         a.d0 = F->d32[0], a.d1 = F->d32[1], a.sync = F->sync;
         a.deg = deg, a.theta = theta, a.delta = delta, a.tol = tol, a.inner_tol = ctx->inner_tol;
@@ -460,15 +463,16 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
     {
         PhaseTimer pt(ctx, PH_SOLVE, s);
         // u = 2E^n - E^{n-1} goes straight into E_next: it is also the solver's starting guess
-        k_newmark_uv<<<ge, kBlock, 0, s>>>(F->edge_fixed, E_cur, E_prev, F->dt * F->dt, F->ne, E_next, F->tmp);
+        const double dt2 = F->dt * F->dt;
+        k_newmark_guess<<<ge, kBlock, 0, s>>>(F->edge_fixed, E_cur, E_prev, F->ne, E_next);
         if (f32)
-            k_newmark_rhs<float><<<ge, kBlock, 0, s>>>(Sell{F->se_ptr, F->se_w, F->se_col}, F->se_M, F->se_S,
-                                                       F->edge_fixed, E_next, F->tmp, (const float*)dG_half,
-                                                       (const float*)dG_prev, F->ne, F->rhs);
+            k_newmark_rhs<float><<<ge, kBlock, 0, s>>>(Sell{F->se_ptr, F->se_w, F->se_col}, F->se_A, F->se_S,
+                                                       F->edge_fixed, E_next, E_cur, dt2, (const float*)dG_half,
+                                                       (const float*)dG_prev, F->ne, F->rhs, F->z);
         else
-            k_newmark_rhs<double><<<ge, kBlock, 0, s>>>(Sell{F->se_ptr, F->se_w, F->se_col}, F->se_M, F->se_S,
-                                                        F->edge_fixed, E_next, F->tmp, (const double*)dG_half,
-                                                        (const double*)dG_prev, F->ne, F->rhs);
+            k_newmark_rhs<double><<<ge, kBlock, 0, s>>>(Sell{F->se_ptr, F->se_w, F->se_col}, F->se_A, F->se_S,
+                                                        F->edge_fixed, E_next, E_cur, dt2, (const double*)dG_half,
+                                                        (const double*)dG_prev, F->ne, F->rhs, F->z);
         FP_CUDA_TRY(ctx, cudaGetLastError());
     }
     // learned correction of the guess (with fallback), and/or collection of its residual
@@ -476,8 +480,11 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
         fp_status sl = learned_guess(ctx, FP_SYS_NEWMARK, F->rhs, E_next, s);
         if (sl != FP_OK) return sl;
     }
-    // Newmark solve for E^N from the guess 2E^n - E^{n-1} (written into E_next above)
-    fp_status st = run_pcg(ctx, FP_SYS_NEWMARK, F->rhs, E_next, tol, nullptr, max_iter, 0, s, F->tmp);
+    // Newmark solve for E^N from the guess 2E^n - E^{n-1} (written into E_next above), whose residual
+    // is known unless the learned correction may have replaced it
+    const bool replaced = learned_active(F, FP_SYS_NEWMARK) && learned_model(F, FP_SYS_NEWMARK) == FP_LEARNED_GUESS;
+    fp_status st = run_pcg(ctx, FP_SYS_NEWMARK, F->rhs, E_next, tol, nullptr, max_iter, 0, s, F->tmp, false,
+                           replaced ? nullptr : F->z);
     if (st != FP_OK) return st;
     // Gauss-law projection: L d = D0^T M E^N + Q on interior nodes, to ||r|| <= tol ||Q||.
     // D0^T M E^N = D0^T A E^N, since D0^T S = (S D0)^T = 0 (curl grad = 0) on the rows the

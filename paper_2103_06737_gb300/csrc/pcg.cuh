@@ -70,6 +70,7 @@ struct ResidentArgs {
     double* px;             // solution in row order (x itself without a permutation)
     double* ax;             // null, or A x for the final x in DOF order
     bool x_zero;            // the start is zero, whatever x holds
+    const double* r0;       // null, or the start's residual, DOF order
     const double* scale_vec;
     double* r64;            // FP64 residual, row order
     float *z, *d0, *d1;     // vectors that products gather, row order
@@ -96,6 +97,7 @@ struct StreamArgs {
     const int32_t* perm;    // row -> DOF (null: rows in DOF order)
     const double* b;        // right-hand side, DOF order
     double* x;              // start and solution, DOF order
+    const double* r0;       // null, or the start's residual, DOF order
     double *pb, *px;        // both in row order (b and x themselves without a permutation)
     double* ax;             // null, or A x for the final x in DOF order
     const double* scale_vec;   // row order (no permutation with it)

@@ -230,7 +230,7 @@ struct Resident {
                 const int row = 32 * (s0 + s) + lane;
                 if (row < a.n) px[row] = a.x_zero ? 0.0 : a.x[a.perm ? __ldg(a.perm + row) : row];
             }
-            if (!a.x_zero && !g.barrier()) return false;
+            if (!a.r0 && !g.barrier()) return false;
         }
         for (;;) {
             // ---- outer residual in FP64
@@ -240,7 +240,7 @@ struct Resident {
                 if (row >= a.n) continue;
                 const int k = a.perm ? __ldg(a.perm + row) : row;
                 const double b = __ldg(a.b + k);
-                const double ri = a.x_zero && outer == 0 ? b : b - sell_row_cached(a.S, a.val, px, row);
+                const double ri = a.r0 && outer == 0 ? __ldg(a.r0 + k) : b - sell_row_cached(a.S, a.val, px, row);
                 a.r64[row] = ri;
                 v[0] += ri * ri;
                 if (outer == 0) {

@@ -360,8 +360,8 @@ struct ResidualRows {        // r64 = b - A x
         double b, s;
     };
     __device__ __forceinline__ Row load(int64_t i) const { return Row{ld_row(a.pb + i), ref && a.scale_vec ? ld_row(a.scale_vec + i) : 0.0}; }
-    __device__ __forceinline__ void apply(int64_t i, const Row& r, double t) {
-        const double ri = r.b - t;
+    __device__ __forceinline__ void apply(int64_t i, const Row& r, double t) { take(i, r, r.b - t); }
+    __device__ __forceinline__ void take(int64_t i, const Row& r, double ri) {
         a.r64[i] = ri;
         rr += ri * ri;
         if (ref) bb += r.b * r.b, ss += r.s * r.s;
@@ -508,15 +508,16 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
         } else if (a.x_zero) {
             for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) a.px[i] = 0.0;
         }
-        if (!a.x_zero) R.start(OP_F64);
+        if (!a.r0) R.start(OP_F64);
         if (!g.barrier()) return false;
         for (;;) {
             // ---- outer residual in FP64
             double v[3];
             {
                 ResidualRows f{a, outer == 0, 0.0, 0.0, 0.0};
-                if (a.x_zero && outer == 0) {   // r = b
-                    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) f.apply(i, f.load(i), 0.0);
+                if (a.r0 && outer == 0) {
+                    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x)
+                        f.take(i, f.load(i), __ldg(a.r0 + (a.perm ? __ldg(a.perm + i) : i)));
                 } else {
                     stream_pass<OP_F64>(R, a.px, f);
                 }
