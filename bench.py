@@ -259,19 +259,20 @@ def pcg_bytes_per_iter(n_rows, nnz, val_bytes=8):
 
 
 def mixed_solve_bytes(n_rows, nnz, inner_iters, outer, deg=1):
-    """Minimal DRAM bytes of one mixed-precision solve: per FP32 inner PCG iteration the FP32
-    operator once (4 B value + 4 B column per nonzero) and 13 FP32 vector passes (update: c,
-    r read+write, p, q, diag^-1 read, z written; search: z, p, q read, p, q written); with a
-    Chebyshev preconditioner of degree deg > 1, per application 5 vector passes to start it (r,
-    diag^-1 read; d, z, s written) and deg - 1 further products with 7 vector passes each (d,
-    s, diag^-1, z read; s, d, z written); per refinement the start of the inner solve (one
-    preconditioner application, one FP32 product, r64 and diag^-1 read, r, z, p, q written)
-    and the FP64 update x += |r| c; outer + 1 FP64 residuals b - A x (12 B per nonzero, b and x
-    read, r64 written, c cleared)."""
-    prec = 0 if deg <= 1 else 5 * 4 * n_rows + (deg - 1) * (nnz * 8 + 7 * 4 * n_rows)
-    inner = inner_iters * (nnz * 8 + 13 * 4 * n_rows + prec)
-    start = outer * (prec + nnz * 8 + (8 + 4 + 4 * 4) * n_rows + (8 + 8 + 4) * n_rows)
-    resid = (outer + 1) * (nnz * 12 + (8 + 8 + 8 + 4) * n_rows)
+    """DRAM bytes of one mixed-precision solve that streams its operators: per FP32 inner PCG
+    iteration the FP32 operator once (4 B value + 2 B column + 1/8 B of base column per nonzero)
+    and 13 FP32 vector passes (update: r read+write, q, diag^-1 read, z written; product: z read,
+    p, q, c read+write); with a Chebyshev preconditioner of degree deg > 1, per application 5
+    vector passes to start it (r, diag^-1 read; d, z, s written) and deg - 1 further products with
+    7 vector passes each (d, s, diag^-1, z read; s, d, z written); per refinement the start of the
+    inner solve (one preconditioner application, one FP32 product, r64 and diag^-1 read, r, z, p,
+    q written) and the FP64 update x += |r| c; outer + 1 FP64 residuals b - A x (10.125 B per
+    nonzero, b and x read, r64 written, c cleared)."""
+    op = nnz * 6.125
+    prec = 0 if deg <= 1 else 5 * 4 * n_rows + (deg - 1) * (op + 7 * 4 * n_rows)
+    inner = inner_iters * (op + 13 * 4 * n_rows + prec)
+    start = outer * (prec + op + (8 + 4 + 4 * 4) * n_rows + (8 + 8 + 4) * n_rows)
+    resid = (outer + 1) * (nnz * 10.125 + (8 + 8 + 8 + 4) * n_rows)
     return inner + start + resid
 
 
@@ -608,7 +609,8 @@ def run_gpu(args):
         if sort_now:
             lib.sort(bufs[k][b_], bufs[k][1 - b_])
             b_ = 1 - b_
-            n_k += 5
+            # count, scan (3), scatter; from 2^17 particles also to and from records
+            n_k += 7 if bufs[k][b_].n >= 1 << 17 else 5
         s_ = bufs[k][b_]
         if k == 0:
             dG.zero_()
@@ -636,10 +638,9 @@ def run_gpu(args):
         if field:                 # fields: Newmark, Gauss-law projection, Faraday -> E^{n+1}, b^{n+1}
             F.fem_pic_field_step(lib.h, E_prev, e, E_next, b, dG, dG_prev, Qn, tol=args.tol,
                                  max_iter=args.max_iter, precond=state["precond"], info=False)
-            # Newmark right-hand side (2) and solve (mixed: gather into its row order, solve,
-            # scatter out with A E^N: 3; FP64: the solve, then M E^N: 2), Gauss right-hand side
-            # (1), solve (1), projection and Faraday update (2)
-            n_k += 9 if solv[0] == "mixed" else 8     # (a learned preconditioner acts inside the solver)
+            # Newmark right-hand side (2) and solve (mixed: 1; FP64: the solve, then M E^N: 2),
+            # Gauss right-hand side with the Faraday update (1), solve (1), projection (1)
+            n_k += 6 if solv[0] == "mixed" else 7     # (a learned preconditioner acts inside the solver)
         lib.residuals(dG, Qn, Qo, b, res)
         n_k += 1
         Qo.copy_(Qn)
@@ -1277,14 +1278,14 @@ def run_gpu(args):
                     model = (mixed_solve_bytes(rows, nz, its, outs, 1 if lrn else main_pdeg[k_sys]) if mixed else
                              pcg_bytes_per_iter(rows, nz) * max(its, 1))
                     if lrn:   # one product with the BF16 learned correction per inner iteration
-                        model += its * nz * 6
-                    op_bytes = nz * 8 * 1.2          # FP32 SELL operator (value + column), ~1.2x padding
+                        model += its * nz * 4.125
+                    op_bytes = nz * 6.125 * 1.2      # FP32 SELL operator (value + packed column), ~1.2x padding
                     on_chip = op_bytes < L2_BYTES
-                    traffic = measured_traffic(("k_pcg_mixed/" if mixed else "k_pcg/") + ph +
+                    traffic = measured_traffic(("k_pcg_stream/" if mixed else "k_pcg/") + ph +
                                                ("/learned" if lrn else ""), wl.name, its)
                     pc_name = ("learned preconditioner" if lrn else
                                f"Chebyshev-Jacobi degree {main_pdeg[k_sys]}" if main_pdeg[k_sys] > 1 else "Jacobi")
-                    name = ("k_pcg_mixed (" + ph.split("_")[1] + f" system, FP32 inner PCG, {pc_name}, FP64 residual)"
+                    name = ("k_pcg_resident or k_pcg_stream (" + ph.split("_")[1] + f" system, FP32 inner PCG, {pc_name}, FP64 residual)"
                             if mixed else "k_pcg (" + ph.split("_")[1] + " system, FP64)")
                     ach = byt / (avg * 1e-3) / 1e9
                     cand.append((avg, {
@@ -1299,7 +1300,7 @@ def run_gpu(args):
                         "rows": rows, "nnz": nz,
                         "model_bytes_per_launch": model,
                         "model_frac": model / (avg * 1e-3) / 1e9 / peak,
-                        "model_rule": ("what the mixed solver moves: the FP32 operator (8 B per nonzero) once per "
+                        "model_rule": ("what the mixed solver moves: the FP32 operator (6.1 B per nonzero) once per "
                                        "product, deg products per inner iteration, FP32 vector passes, FP64 "
                                        "residuals per refinement" if mixed else "FP64 PCG, 12 B per nonzero + "
                                        "13 FP64 vector passes per iteration"),
