@@ -53,7 +53,7 @@ typedef enum {
     FP_EINVAL = 1,   /* bad argument, size or pointer; invalid cell id; non-finite particle state */
     FP_ECUDA = 2,    /* a CUDA runtime call failed (text in fem_pic_last_error) */
     FP_EWALK = 3,    /* a particle hit the crossing bound of the tet walk */
-    FP_ENOCONV = 4,  /* an iterative solve reached its iteration cap */
+    FP_ENOCONV = 4,  /* an iterative solve reached its iteration cap, or its residual is no finite number */
     FP_EGEOM = 5     /* a tet with zero volume, or a non-manifold face */
 } fp_status;
 
@@ -375,7 +375,8 @@ fp_status fem_pic_field_matrix(const fem_pic_t* ctx, int which, int32_t* row_ptr
  * Jacobi-preconditioned CG (precond, see FP_PC_*), starting from the x passed in (device, in/out),
  * until ||rhs - A x|| <= tol ||rhs|| or max_iter iterations.  rhs must be zero on PEC
  * rows.  info (host, may be NULL) is filled after a stream synchronisation; with info
- * a solve that stops at max_iter returns FP_ENOCONV, otherwise the status word records it.
+ * a solve that stops at max_iter, or whose residual is no finite number (NaN or infinite
+ * inputs, squares beyond the FP64 range), returns FP_ENOCONV, otherwise the status word records it.
  */
 fp_status fem_pic_field_solve(fem_pic_t* ctx, int system, const double* rhs, double* x, double tol,
                               int max_iter, int precond, fp_solve_info* info, void* stream);

@@ -495,7 +495,7 @@ fp_status fem_pic_status(fem_pic_t* ctx, void* stream) {
         return FP_EWALK;
     }
     if (h & ST_NOCONV) {
-        ctx->err = "an iterative field solve reached its iteration cap";
+        ctx->err = "an iterative field solve reached its iteration cap, or its residual was no finite number";
         return FP_ENOCONV;
     }
     return FP_OK;

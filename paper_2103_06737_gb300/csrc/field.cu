@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(BS, BS >= 1024 ? 1 : kSolverPerSm) k_pcg(PcgAr
         a.out[1] = rr;
         a.out[2] = bb;      // squared norm the residual is measured against
         a.out[3] = 0.0;
-        if (rr > thr) atomicOr(a.status, ST_NOCONV);
+        if (!solve_met(rr, thr)) atomicOr(a.status, ST_NOCONV);
     }
 }
 
@@ -373,15 +373,14 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
     return FP_OK;
 }
 
-fp_status fill_info(fem_pic* ctx, int slot, fp_solve_info* info, cudaStream_t s, float ms) {
+// tol: the tolerance the solve had (FP_ENOCONV where it missed it); below 0: only the numbers
+fp_status fill_info(fem_pic* ctx, int slot, double tol, fp_solve_info* info, cudaStream_t s, float ms) {
     if (!info) return FP_OK;
     double o[4];
     FP_CUDA_TRY(ctx, cudaMemcpyAsync(o, ctx->field->out + 4 * slot, sizeof o, cudaMemcpyDeviceToHost, s));
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    info->iters = (int32_t)o[0];
-    info->outer = (int32_t)o[3];
-    info->rel_res = o[2] > 0 ? sqrt(o[1] / o[2]) : sqrt(o[1]);
-    info->abs_res = sqrt(o[1]);
+    fp_status met = solve_outcome(o, tol, info);
+    if (tol < 0.0 && met == FP_ENOCONV) met = FP_OK;
     info->ms = ms;
     info->precond = ctx->field->last_fp64[slot] ? FP_PC_JACOBI_FP64 : FP_PC_JACOBI;
     info->fell_back = 0;
@@ -393,7 +392,7 @@ fp_status fill_info(fem_pic* ctx, int slot, fp_solve_info* info, cudaStream_t s,
         info->precond = FP_PC_LEARNED;
         info->fell_back = fl;
     }
-    return FP_OK;
+    return met;
 }
 
 // Natural boundary (Eq. zero_mean_constraint): the projection solves L d = g - (sum g / sum
@@ -902,8 +901,8 @@ fp_status fem_pic_field_poly(fem_pic_t* ctx, int system, int degree, double rati
 fp_status fem_pic_field_last_info(fem_pic_t* ctx, fp_solve_info info[2], void* stream) {
     if (!ctx || !ctx->field || !info) return FP_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    fp_status st = fill_info(ctx, 0, &info[0], s, 0.f);
-    if (st == FP_OK) st = fill_info(ctx, 1, &info[1], s, 0.f);
+    fp_status st = fill_info(ctx, 0, -1.0, &info[0], s, 0.f);
+    if (st == FP_OK) st = fill_info(ctx, 1, -1.0, &info[1], s, 0.f);
     return st;
 }
 
@@ -977,8 +976,7 @@ fp_status fem_pic_field_solve(fem_pic_t* ctx, int system, const double* rhs, dou
         cudaEventRecord(b, s);
         cudaEventSynchronize(b);
         cudaEventElapsedTime(&ms, a, b);
-        st = fill_info(ctx, 0, info, s, ms);
-        if (st == FP_OK && info->rel_res > tol) st = FP_ENOCONV;
+        st = fill_info(ctx, 0, tol, info, s, ms);
     }
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
@@ -1010,10 +1008,9 @@ fp_status fem_pic_field_step(fem_pic_t* ctx, const double* E_prev, const double*
     cudaStream_t s = (cudaStream_t)stream;
     fp_status st = field_step_impl(ctx, E_prev, E_cur, E_next, b, dG_half, dG_prev, Q_new, tol, max_iter, s);
     if (st != FP_OK || !info) return st;
-    st = fill_info(ctx, 0, &info[0], s, 0.f);
-    if (st == FP_OK) st = fill_info(ctx, 1, &info[1], s, 0.f);
-    if (st == FP_OK && (info[0].rel_res > tol || info[1].rel_res > tol)) st = FP_ENOCONV;
-    return st;
+    st = fill_info(ctx, 0, tol, &info[0], s, 0.f);
+    const fp_status gs = fill_info(ctx, 1, tol, &info[1], s, 0.f);
+    return st != FP_OK && (st != FP_ENOCONV || gs == FP_OK) ? st : gs;   // the graver of the two
 }
 
 fp_status fem_pic_field_initial(fem_pic_t* ctx, const void* Q, double* E, double tol, int max_iter,
@@ -1043,8 +1040,7 @@ fp_status fem_pic_field_initial(fem_pic_t* ctx, const void* Q, double* E, double
     k_project<<<ge, kBlock, 0, s>>>(ctx->d_edges, F->edge_fixed, F->delta, F->tmp, F->ne, E);
     FP_CUDA_TRY(ctx, cudaGetLastError());
     if (info) {
-        st = fill_info(ctx, 1, info, s, 0.f);
-        if (st == FP_OK && info->rel_res > tol) st = FP_ENOCONV;
+        st = fill_info(ctx, 1, tol, info, s, 0.f);
     }
     return st;
 }

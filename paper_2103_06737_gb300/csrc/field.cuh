@@ -3,6 +3,8 @@
 
 #include <cuda_bf16.h>
 
+#include <cfloat>
+
 #include "internal.cuh"
 
 namespace fempic {
@@ -25,6 +27,14 @@ double jacobi_lambda_max(const std::vector<int32_t>& rp, const std::vector<int32
                          const std::vector<double>& val, int steps);
 
 struct LearnedDev;  // learned correction (learned.cu)
+
+// A solve that ended with a squared residual norm rr has met its threshold.  Not where the residual is
+// no finite number: such a solve stops (nothing is left to reduce) but has no solution.
+__host__ __device__ inline bool solve_met(double rr, double thr) { return rr <= thr && rr <= DBL_MAX; }
+
+// What a solve's output words (iterations, |r|^2, |reference|^2, refinements) say: the numbers of info,
+// and FP_OK, or FP_ENOCONV where the relative residual is not within tol (NaN included).
+fp_status solve_outcome(const double out[4], double tol, fp_solve_info* info);
 
 // launch shape of the on-chip mixed solver for one system (pcg_resident.cu)
 struct ResidentPlan {

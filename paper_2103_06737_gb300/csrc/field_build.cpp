@@ -13,6 +13,14 @@
 
 namespace fempic {
 
+fp_status solve_outcome(const double out[4], double tol, fp_solve_info* info) {
+    info->iters = (int32_t)out[0];
+    info->outer = (int32_t)out[3];
+    info->rel_res = out[2] > 0 ? std::sqrt(out[1] / out[2]) : std::sqrt(out[1]);
+    info->abs_res = std::sqrt(out[1]);
+    return info->rel_res <= tol ? FP_OK : FP_ENOCONV;
+}
+
 namespace {
 
 const int kLE[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};

@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
         a.out[1] = f.rr;
         a.out[2] = f.ref2;
         a.out[3] = (double)outer;
-        if (f.rr > f.thr) atomicOr(a.status, ST_NOCONV);
+        if (!solve_met(f.rr, f.thr)) atomicOr(a.status, ST_NOCONV);
     }
 }
 

@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
         a.out[1] = ref.rr;
         a.out[2] = ref.ref2;
         a.out[3] = (double)outer;
-        if (ref.rr > ref.thr) atomicOr(a.status, ST_NOCONV);
+        if (!solve_met(ref.rr, ref.thr)) atomicOr(a.status, ST_NOCONV);
     }
 }
 

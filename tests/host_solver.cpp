@@ -1,0 +1,19 @@
+// Host-side decisions of the field solvers with a small C interface.  Test infrastructure: built by
+// tests/test_host_solver.py with g++.
+#include "../paper_2103_06737_gb300/csrc/field.cuh"
+
+using namespace fempic;
+
+extern "C" {
+
+// the status and {rel_res, abs_res, iters, outer} that a solve's output words stand for
+int hs_outcome(const double* out, double tol, double* r) {
+    fp_solve_info info{};
+    const int st = (int)solve_outcome(out, tol, &info);
+    r[0] = info.rel_res, r[1] = info.abs_res, r[2] = info.iters, r[3] = info.outer;
+    return st;
+}
+
+int hs_met(double rr, double thr) { return solve_met(rr, thr) ? 1 : 0; }
+
+}  // extern "C"

@@ -1,0 +1,44 @@
+"""A field solve that ends without a solution says so: in the returned status where info is asked
+for, in the status word where it is not."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2103_06737_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+F = pytest.importorskip("paper_2103_06737_gb300.fem_pic")
+
+
+def _lib(n):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    m = I.cube_mesh(n, 1.0, 0.1, seed=1)
+    lib = F.FemPic(m.xyz, m.tets, F.FP_FP32)
+    F.fem_pic_field_setup(lib.h, 0.2 * I.gyro_period(0.1))
+    return lib
+
+
+# one block, on chip over several blocks, streamed; and the FP64 solver
+@pytest.mark.parametrize("n,pc", [(2, F.FP_PC_JACOBI), (9, F.FP_PC_JACOBI), (36, F.FP_PC_JACOBI),
+                                  (9, F.FP_PC_JACOBI_FP64)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), 1e200])
+def test_no_finite_residual_is_no_convergence(n, pc, bad):
+    lib = _lib(n)
+    rp, _, _ = F.fem_pic_field_matrix(lib.h, 2)
+    rhs = torch.zeros(lib.n_edges, dtype=torch.float64, device="cuda")
+    rhs[int(np.nonzero(np.diff(rp) > 1)[0][0])] = bad
+    x = torch.zeros_like(rhs)
+    st, info = F.fem_pic_field_solve(lib.h, F.FP_SYS_NEWMARK, rhs, x, tol=1e-10, precond=pc)
+    assert st == F.FP_ENOCONV and not info["rel_res"] <= 1e-10 and info["iters"] == 0
+    assert lib.status() == F.FP_ENOCONV
+    x.zero_()
+    F.fem_pic_field_solve(lib.h, F.FP_SYS_NEWMARK, rhs, x, tol=1e-10, precond=pc, info=False)
+    assert lib.status() == F.FP_ENOCONV
+    rhs.zero_()
+    x.zero_()
+    st, info = F.fem_pic_field_solve(lib.h, F.FP_SYS_NEWMARK, rhs, x, tol=1e-10, precond=pc)
+    assert st == F.FP_OK and info["rel_res"] == 0.0 and float(x.abs().max()) == 0.0
+    assert lib.status() == F.FP_OK
+    lib.close()

@@ -1,0 +1,43 @@
+"""Host-side decisions of the field solvers, on the library's own source compiled with g++."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from test_host_assembly import CSRC, HERE, ROOT, _cuda_include
+
+OK, ECUDA, ENOCONV = 0, 2, 4
+INF, NAN = float("inf"), float("nan")
+
+
+@pytest.fixture(scope="module")
+def hs(tmp_path_factory):
+    cxx, inc = shutil.which("g++"), _cuda_include()
+    if not cxx or not inc:
+        pytest.skip("needs g++ and the CUDA headers")
+    out = str(tmp_path_factory.mktemp("hs") / "libhs.so")
+    cmd = [cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I" + inc, "-I" + os.path.join(ROOT, "include"),
+           os.path.join(HERE, "host_solver.cpp"), os.path.join(CSRC, "field_build.cpp"), "-o", out]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    lib = ctypes.CDLL(out)
+    lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
+    lib.hs_met.argtypes = [ctypes.c_double, ctypes.c_double]
+    return lib
+
+
+# iterations, |r|^2, |reference|^2, refinements -> status at a tolerance of 1e-10
+@pytest.mark.parametrize("words,status", [
+    ((12, 1e-22, 1.0, 2), OK), ((0, 0.0, 0.0, 0), OK),             # within it; a zero right-hand side
+    ((9, 1e-18, 1.0, 2), ENOCONV),                                  # the iteration cap
+    ((0, NAN, 1.0, 0), ENOCONV), ((0, NAN, NAN, 0), ENOCONV),       # a NaN in the start, in the right-hand side
+    ((0, INF, 1.0, 0), ENOCONV), ((0, INF, INF, 0), ENOCONV)])      # a norm that overflows
+def test_outcome_of_a_solve(hs, words, status):
+    w, r = np.array(words, np.float64), np.zeros(4)
+    assert hs.hs_outcome(w.ctypes.data, 1e-10, r.ctypes.data) == status
+    assert (r[2], r[3]) == (words[0], words[3])
+    # the device sets the status word's bit by the same rule
+    assert hs.hs_met(w[1], 1e-20 * w[2]) == (status == OK)
