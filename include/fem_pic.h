@@ -377,6 +377,9 @@ fp_status fem_pic_field_matrix(const fem_pic_t* ctx, int which, int32_t* row_ptr
  * rows.  info (host, may be NULL) is filled after a stream synchronisation; with info
  * a solve that stops at max_iter, or whose residual is no finite number (NaN or infinite
  * inputs, squares beyond the FP64 range), returns FP_ENOCONV, otherwise the status word records it.
+ * The mixed solvers run on all SMs together and bound their waits for each other: a solve that
+ * gives up returns FP_ECUDA with info (x is then unspecified), the status word records it, and the
+ * handle's further mixed solves give up at once until fem_pic_status has reported it.
  */
 fp_status fem_pic_field_solve(fem_pic_t* ctx, int system, const double* rhs, double* x, double tol,
                               int max_iter, int precond, fp_solve_info* info, void* stream);
@@ -600,9 +603,10 @@ fp_status fem_pic_profile_read(fem_pic_t* ctx, double ms[16], int64_t count[16],
  * Self-test of the failure path of the library's bounded waits (not part of the method; the
  * paper has no counterpart): a one-thread kernel waits on a barrier that nothing completes,
  * gives up after limit_s seconds (0 < limit_s <= 10, else FP_EINVAL) and sets the time-out
- * bit of the status word, exactly as a push kernel does when a bulk copy never lands; the
- * next fem_pic_status returns FP_ECUDA and clears it, and the context stays usable.  Nothing
- * faults or hangs.  Asynchronous.
+ * bit of the status word, exactly as a push kernel does when a bulk copy never lands; after
+ * fem_pic_field_setup a second kernel gives up likewise on an exchange of the field solvers
+ * that no other block joins (see fem_pic_field_solve).  The next fem_pic_status returns FP_ECUDA
+ * and clears both, and the context stays usable.  Nothing faults or hangs.  Asynchronous.
  */
 fp_status fem_pic_selftest_wait(fem_pic_t* ctx, double limit_s, void* stream);
 

@@ -465,7 +465,8 @@ fp_status fem_pic_selftest_wait(fem_pic_t* ctx, double limit_s, void* stream) {
         if (ctx) ctx->err = "fem_pic_selftest_wait: limit outside (0, 10] s";
         return FP_EINVAL;
     }
-    return launch_wait_selftest(ctx, limit_s, (cudaStream_t)stream);
+    const fp_status st = launch_wait_selftest(ctx, limit_s, (cudaStream_t)stream);
+    return st != FP_OK ? st : launch_exchange_selftest(ctx, limit_s, (cudaStream_t)stream);
 }
 
 fp_status fem_pic_status(fem_pic_t* ctx, void* stream) {
@@ -476,9 +477,11 @@ fp_status fem_pic_status(fem_pic_t* ctx, void* stream) {
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     FP_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_status, 0, 4, s));
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    if (h & ST_TIMEOUT) {
+    if (h & (ST_TIMEOUT | ST_EXCHANGE)) {
         FP_CUDA_TRY(ctx, field_reset_sync(ctx, s));
-        ctx->err = "a kernel gave up waiting for its asynchronous copies";
+        ctx->err = (h & ST_TIMEOUT) ? "a kernel gave up waiting for its asynchronous copies"
+                                    : "a field solve gave up waiting for its other blocks: its solution and those of "
+                                      "the solves since are not valid";
         return FP_ECUDA;
     }
     if (h & ST_NONFINITE) {

@@ -381,6 +381,7 @@ fp_status fill_info(fem_pic* ctx, int slot, double tol, fp_solve_info* info, cud
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     fp_status met = solve_outcome(o, tol, info);
     if (tol < 0.0 && met == FP_ENOCONV) met = FP_OK;
+    if (met == FP_ECUDA) ctx->err = "a field solve gave up waiting for its other blocks: no solution (fem_pic_status resets it)";
     info->ms = ms;
     info->precond = ctx->field->last_fp64[slot] ? FP_PC_JACOBI_FP64 : FP_PC_JACOBI;
     info->fell_back = 0;
@@ -528,7 +529,23 @@ fp_status field_step_impl(fem_pic_t* ctx, const double* E_prev, const double* E_
 
 }  // namespace
 
-// after a wait of the on-chip solver ran out: the words of its grid exchanges start afresh
+// a block that joins an exchange of two and is alone in it
+static __global__ void k_exchange_selftest(void* sync, int32_t* status, uint64_t limit_ns) {
+    __shared__ GridSyncShared sh;
+    GridSync<false> g;
+    g.init(sync, &sh, status);
+    g.nb = 2;
+    g.limit = limit_ns;
+    g.barrier();
+}
+fp_status launch_exchange_selftest(fem_pic* ctx, double limit_s, cudaStream_t s) {
+    if (!ctx->field || !ctx->field->sync) return FP_OK;
+    k_exchange_selftest<<<1, 32, 0, s>>>(ctx->field->sync, ctx->d_status, (uint64_t)(limit_s * 1e9));
+    FP_CUDA_TRY(ctx, cudaGetLastError());
+    return FP_OK;
+}
+
+// after a wait of a mixed solver ran out: the words of its grid exchanges start afresh
 cudaError_t field_reset_sync(fem_pic* ctx, cudaStream_t s) {
     if (!ctx->field || !ctx->field->sync) return cudaSuccess;
     return cudaMemsetAsync(ctx->field->sync, 0, grid_sync_bytes(ctx->sm_count), s);

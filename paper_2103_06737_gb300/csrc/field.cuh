@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <cfloat>
+#include <cmath>
 
 #include "internal.cuh"
 
@@ -33,7 +34,13 @@ struct LearnedDev;  // learned correction (learned.cu)
 __host__ __device__ inline bool solve_met(double rr, double thr) { return rr <= thr && rr <= DBL_MAX; }
 
 // What a solve's output words (iterations, |r|^2, |reference|^2, refinements) say: the numbers of info,
-// and FP_OK, or FP_ENOCONV where the relative residual is not within tol (NaN included).
+// and FP_OK, or FP_ENOCONV where the relative residual is not within tol (NaN included).  FP_ECUDA
+// where the refinements still are kAbandoned: a mixed solver writes {0, infinity, 1, kAbandoned} when
+// it starts, so that one that gives up does not leave an earlier solve's numbers.
+constexpr double kAbandoned = -1.0;
+__host__ __device__ inline void solve_begin(double out[4]) {
+    out[0] = 0.0, out[1] = HUGE_VAL, out[2] = 1.0, out[3] = kAbandoned;
+}
 fp_status solve_outcome(const double out[4], double tol, fp_solve_info* info);
 
 // launch shape of the on-chip mixed solver for one system (pcg_resident.cu)

@@ -20,9 +20,10 @@
 // mailbox of partials per block, measured 2.7-5 us: 152 blocks' words per exchange are more
 // traffic than the trip they save.)
 //
-// Every wait is bounded: a block that does not see the others within kGridWaitNs sets ST_TIMEOUT
-// in the status word and leaves (all its threads together); the others follow, and
-// fem_pic_status clears the words.
+// Every wait is bounded: a block that does not see the others within kGridWaitNs sets ST_EXCHANGE
+// in the status word and a mark beside the words, and leaves (all its threads together); the
+// others see the mark and follow.  The words then hold arrivals that belong to no exchange, so a
+// launch that finds the mark leaves at its first exchange; fem_pic_status clears words and mark.
 #pragma once
 
 #include "async_copy.cuh"
@@ -31,10 +32,10 @@
 namespace fempic {
 
 constexpr uint64_t kGridWaitNs = 2000000000ull;      // 2 s
-// device memory of one handle's exchanges (zeroed at setup): the words at rest, the words
-// in use (two exchanges; a line each), then the blocks' partials for the sums that
-// are added one by one (two copies of three doubles per block)
-constexpr size_t kGridLine = 128;
+// device memory of one handle's exchanges (zeroed at setup): the words at rest and the mark of an
+// abandoned exchange, the words in use (two exchanges; a line each), then the blocks' partials for
+// the sums that are added one by one (two copies of three doubles per block)
+constexpr size_t kGridLine = 128, kGridMark = 64;
 inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * blocks * 3 * 8; }
 
 #ifdef __CUDACC__
@@ -44,7 +45,7 @@ struct GridSyncShared {
     float part[2][3][33];        // per-warp partials, by the exchange's parity
     float tot[2][2];
     unsigned long long prev[2][2];   // what each word held after this block's last exchange on it
-    int fail;                    // set by a thread whose own wait ran out: the block does not arrive any more
+    int fail;                    // the block does not arrive any more: its own wait ran out, or the mark is set
     int state[2];                // bit 0: a wait ran out, bit 1: add the partials one by one
 };
 
@@ -53,6 +54,7 @@ struct GridSync {
     char* mem;
     GridSyncShared* sh;
     int32_t* status;
+    uint64_t limit;            // of a wait, ns
     uint32_t turn;             // exchanges so far
     int nb, lane, wid, warps;
 
@@ -60,6 +62,7 @@ struct GridSync {
         mem = static_cast<char*>(m);
         sh = s;
         status = st;
+        limit = kGridWaitNs;
         turn = 0;
         nb = gridDim.x;
         lane = threadIdx.x & 31;
@@ -68,8 +71,14 @@ struct GridSync {
         // nothing changes the words at rest before every block's first arrival
         if (!ONE && threadIdx.x < 4) s->prev[threadIdx.x >> 1][threadIdx.x & 1] =
             *reinterpret_cast<volatile unsigned long long*>(mem + 8 * threadIdx.x);
-        if (threadIdx.x == 0) s->fail = 0;
+        if (threadIdx.x == 4) s->fail = ONE ? 0 : *mark();
         __syncthreads();
+    }
+    __device__ __forceinline__ volatile int* mark() { return reinterpret_cast<volatile int*>(mem + kGridMark); }
+    // one thread: the exchange is abandoned
+    __device__ __forceinline__ void abandon() {
+        atomicOr(status, ST_EXCHANGE);
+        *mark() = 1;
     }
     // by one thread at the end of a launch whose waits all ended: the next launch starts here
     __device__ __forceinline__ void finish() {
@@ -113,7 +122,7 @@ struct GridSync {
             }
             if ((spin & 1023u) == 1023u) {
                 if (t0 == 0) t0 = global_ns();
-                if (global_ns() - t0 > kGridWaitNs) return false;
+                if (*mark() != 0 || global_ns() - t0 > limit) return false;
             }
         }
     }
@@ -136,7 +145,7 @@ struct GridSync {
             const unsigned long long q[1] = {1ull};
             unsigned long long d[1];
             const bool ok = !sh->fail && arrive_wait<1>(par, q, d);
-            if (!ok) atomicOr(status, ST_TIMEOUT);
+            if (!ok) abandon();
             sh->state[par] = ok ? 0 : 1;
         }
         __syncthreads();
@@ -187,7 +196,7 @@ struct GridSync {
                 exact = exact || ((d[k] >> 8) & 255ull) != 0 || (t < 16777216ll && t > -16777216ll);
                 sh->tot[par][k] = __ll2float_rn(t) * pow2(-e[k]);
             }
-            if (!ok) atomicOr(status, ST_TIMEOUT);
+            if (!ok) abandon();
             sh->state[par] = ok ? (exact ? 2 : 0) : 1;
         }
         __syncthreads();

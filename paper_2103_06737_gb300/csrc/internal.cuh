@@ -53,7 +53,8 @@ static_assert(sizeof(TetHot) == 128, "TetHot layout");
 // bits of the device status word
 // ST_NONFINITE: a particle's position or velocity (given, or after its push) was not finite;
 // the particle was removed (cell -1) with nothing deposited
-enum : int32_t { ST_WALK = 1, ST_INVAL = 2, ST_NOCONV = 4, ST_TIMEOUT = 8, ST_NONFINITE = 16 };
+// ST_EXCHANGE: a field solve's blocks lost each other, its solution is not valid
+enum : int32_t { ST_WALK = 1, ST_INVAL = 2, ST_NOCONV = 4, ST_TIMEOUT = 8, ST_NONFINITE = 16, ST_EXCHANGE = 32 };
 
 struct HostComplex {
     int64_t nn = 0, ne = 0, nf = 0, nt = 0;
@@ -81,6 +82,8 @@ namespace fempic {
 struct FieldDev;
 void field_free(fem_pic* ctx);
 cudaError_t field_reset_sync(fem_pic* ctx, cudaStream_t s);
+// an exchange of the field solvers that another block never joins (nothing without a field setup)
+fp_status launch_exchange_selftest(fem_pic* ctx, double limit_s, cudaStream_t s);
 // phases timed by the optional profiler (fem_pic_profile_*)
 enum Phase : int { PH_PREP = 0, PH_FAST = 1, PH_WALK = 2, PH_PUSH64 = 3, PH_CHARGE = 4, PH_SORT = 5,
                    PH_RESID = 6, PH_SOLVE = 7, PH_CG_NEWMARK = 8, PH_CG_GAUSS = 9, PH_LEARNED = 10,

@@ -316,6 +316,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_pcg_resident(ResidentArgs a) {
     __shared__ GridSyncShared shs;
     __shared__ int sp[kResMaxSlices + 1];
     __shared__ Refinement f;
+    if (!ONE && blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) solve_begin(a.out);   // (one block does not give up)
     GridSync<ONE> g;
     g.init(a.sync, &shs, a.status);
     Resident<THREADS, ONE> S{a, g};

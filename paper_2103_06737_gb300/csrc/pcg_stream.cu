@@ -372,6 +372,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ GridSyncShared shs;
     __shared__ __align__(8) uint64_t full[kStreamBars], empty[kStreamBars];
+    if (blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) solve_begin(a.out);
     GridSync<false> g;
     g.init(a.sync, &shs, a.status);
     const int lane = g.lane, warp = g.wid;

@@ -42,3 +42,35 @@ def test_no_finite_residual_is_no_convergence(n, pc, bad):
     assert st == F.FP_OK and info["rel_res"] == 0.0 and float(x.abs().max()) == 0.0
     assert lib.status() == F.FP_OK
     lib.close()
+
+
+# on chip over several blocks, streamed
+@pytest.mark.parametrize("n", [9, 36])
+def test_abandoned_exchange_is_reported_and_reset(n):
+    """An exchange that a block leaves unfinished: the solves after it give up at once and say so
+    (not with the numbers of the solve before), and fem_pic_status puts the handle back."""
+    lib = _lib(n)
+    rp, col, val = F.fem_pic_field_matrix(lib.h, 2)
+    rhs = np.random.default_rng(n).uniform(-1.0, 1.0, lib.n_edges)
+    rhs[np.diff(rp) == 1] = 0.0
+    rhs = torch.as_tensor(rhs, device="cuda")
+    vec = lambda k: torch.zeros(k, dtype=torch.float64, device="cuda")
+    solve = lambda x, **kw: F.fem_pic_field_solve(lib.h, F.FP_SYS_NEWMARK, rhs, x, tol=1e-10, **kw)
+    x0 = vec(lib.n_edges)
+    st, info = solve(x0)
+    assert st == F.FP_OK and info["iters"] > 0
+    F.fem_pic_selftest_wait(lib.h, 1e-3)
+    with pytest.raises(F.FemPicError, match="gave up waiting"):
+        solve(vec(lib.n_edges))
+    solve(vec(lib.n_edges), info=False)
+    E = [vec(lib.n_edges) for _ in range(3)]
+    with pytest.raises(F.FemPicError, match="gave up waiting"):
+        F.fem_pic_field_step(lib.h, E[0], E[1], E[2], None, None, None,
+                             torch.zeros(lib.n_nodes, dtype=torch.float32, device="cuda"), tol=1e-10)
+    assert lib.status() == F.FP_ECUDA and lib.status() == F.FP_OK
+    x1 = vec(lib.n_edges)
+    st, again = solve(x1)
+    assert st == F.FP_OK and torch.equal(x0, x1)
+    assert (again["iters"], again["outer"], again["rel_res"]) == (info["iters"], info["outer"], info["rel_res"])
+    assert lib.status() == F.FP_OK
+    lib.close()

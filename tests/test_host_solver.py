@@ -34,10 +34,11 @@ def hs(tmp_path_factory):
     ((12, 1e-22, 1.0, 2), OK), ((0, 0.0, 0.0, 0), OK),             # within it; a zero right-hand side
     ((9, 1e-18, 1.0, 2), ENOCONV),                                  # the iteration cap
     ((0, NAN, 1.0, 0), ENOCONV), ((0, NAN, NAN, 0), ENOCONV),       # a NaN in the start, in the right-hand side
-    ((0, INF, 1.0, 0), ENOCONV), ((0, INF, INF, 0), ENOCONV)])      # a norm that overflows
+    ((0, INF, 1.0, 0), ENOCONV), ((0, INF, INF, 0), ENOCONV),       # a norm that overflows
+    ((0, INF, 1.0, -1), ECUDA)])                                    # as a solve writes them when it starts
 def test_outcome_of_a_solve(hs, words, status):
     w, r = np.array(words, np.float64), np.zeros(4)
     assert hs.hs_outcome(w.ctypes.data, 1e-10, r.ctypes.data) == status
-    assert (r[2], r[3]) == (words[0], words[3])
+    assert (r[2], r[3]) == (words[0], max(words[3], 0))
     # the device sets the status word's bit by the same rule
     assert hs.hs_met(w[1], 1e-20 * w[2]) == (status == OK)
