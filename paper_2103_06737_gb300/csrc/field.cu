@@ -535,7 +535,7 @@ static __global__ void k_exchange_selftest(void* sync, int32_t* status, uint64_t
     GridSync<false> g;
     g.init(sync, &sh, status);
     g.nb = 2;
-    g.limit = limit_ns;
+    g.limit1 = limit_ns;
     g.barrier();
 }
 fp_status launch_exchange_selftest(fem_pic* ctx, double limit_s, cudaStream_t s) {

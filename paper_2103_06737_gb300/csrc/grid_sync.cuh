@@ -20,18 +20,22 @@
 // mailbox of partials per block, measured 2.7-5 us: 152 blocks' words per exchange are more
 // traffic than the trip they save.)
 //
-// Every wait is bounded: a block that does not see the others within kGridWaitNs sets ST_EXCHANGE
-// in the status word and a mark beside the words, and leaves (all its threads together); the
-// others see the mark and follow.  The words then hold arrivals that belong to no exchange, so a
-// launch that finds the mark leaves at its first exchange; fem_pic_status clears words and mark.
+// Every wait is bounded: a block that does not see the others within the limit sets ST_EXCHANGE in
+// the status word and a mark beside the words, and leaves (all its threads together); the others
+// see the mark and follow.  The words then hold arrivals that belong to no exchange, so a launch
+// that finds the mark leaves at its first exchange; fem_pic_status clears words and mark.
 #pragma once
 
-#include "async_copy.cuh"
 #include "internal.cuh"
+#ifdef __CUDACC__
+#include "async_copy.cuh"
+#endif
 
 namespace fempic {
 
-constexpr uint64_t kGridWaitNs = 2000000000ull;      // 2 s
+// Limit of a wait.  A launch's first exchange also waits for blocks that have not started because a
+// kernel of another stream still holds their SMs (30 s); the later ones only for blocks at work (2 s).
+constexpr uint64_t kGridStartNs = 30000000000ull, kGridWaitNs = 2000000000ull;
 // device memory of one handle's exchanges (zeroed at setup): the words at rest and the mark of an
 // abandoned exchange, the words in use (two exchanges; a line each), then the blocks' partials for
 // the sums that are added one by one (two copies of three doubles per block)
@@ -54,7 +58,7 @@ struct GridSync {
     char* mem;
     GridSyncShared* sh;
     int32_t* status;
-    uint64_t limit;            // of a wait, ns
+    uint64_t limit, limit1;    // of a wait, ns; of the first
     uint32_t turn;             // exchanges so far
     int nb, lane, wid, warps;
 
@@ -63,6 +67,7 @@ struct GridSync {
         sh = s;
         status = st;
         limit = kGridWaitNs;
+        limit1 = kGridStartNs;
         turn = 0;
         nb = gridDim.x;
         lane = threadIdx.x & 31;
@@ -122,7 +127,7 @@ struct GridSync {
             }
             if ((spin & 1023u) == 1023u) {
                 if (t0 == 0) t0 = global_ns();
-                if (*mark() != 0 || global_ns() - t0 > limit) return false;
+                if (*mark() != 0 || global_ns() - t0 > (turn == 1 ? limit1 : limit)) return false;
             }
         }
     }

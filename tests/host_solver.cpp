@@ -1,6 +1,7 @@
 // Host-side decisions of the field solvers with a small C interface.  Test infrastructure: built by
 // tests/test_host_solver.py with g++.
 #include "../paper_2103_06737_gb300/csrc/field.cuh"
+#include "../paper_2103_06737_gb300/csrc/grid_sync.cuh"
 
 using namespace fempic;
 
@@ -15,5 +16,7 @@ int hs_outcome(const double* out, double tol, double* r) {
 }
 
 int hs_met(double rr, double thr) { return solve_met(rr, thr) ? 1 : 0; }
+
+double hs_wait_seconds(int first) { return 1e-9 * (double)(first ? kGridStartNs : kGridWaitNs); }
 
 }  // extern "C"

@@ -25,6 +25,7 @@ def hs(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(out)
     lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
+    lib.hs_wait_seconds.restype = ctypes.c_double
     lib.hs_met.argtypes = [ctypes.c_double, ctypes.c_double]
     return lib
 
@@ -42,3 +43,10 @@ def test_outcome_of_a_solve(hs, words, status):
     assert (r[2], r[3]) == (words[0], max(words[3], 0))
     # the device sets the status word's bit by the same rule
     assert hs.hs_met(w[1], 1e-20 * w[2]) == (status == OK)
+
+
+def test_first_exchange_waits_for_blocks_that_start_late(hs):
+    """A block can start only when a kernel of another stream has left its SM: the wait for all blocks
+    to be there is many times the wait for blocks at work, and still bounded."""
+    assert 2.0 <= hs.hs_wait_seconds(0) <= 5.0
+    assert 10.0 * hs.hs_wait_seconds(0) <= hs.hs_wait_seconds(1) <= 60.0
