@@ -9,10 +9,11 @@
 //
 //   bits 0-7 arrivals, 8-15 blocks whose partial does not fit, 16-63 signed sum of the partials
 //   scaled by a power of two that all blocks choose alike from the sum's previous values, so
-//   that the expected total lies near 2^32: partials below 2^39 fit, and a total of at least
-//   2^24 is resolved as finely as a float.  Otherwise (a sum that grew or fell more than that,
-//   a value that is not finite) all blocks see it and add the floats themselves, in block
-//   order, behind a second barrier.
+//   that the expected total lies near 2^36: partials below 2^39 fit, and the roundings of at most
+//   255 partials, half a unit each, stay below 2^-24 of a total of at least 2^31, a float's own
+//   rounding.  Otherwise (a sum that grew or fell more than that, a value that is not
+//   finite) all blocks see it in the same word and add the floats, which came with the
+//   exchange, themselves in block order.
 //
 // Words are never cleared: a block subtracts what the word held at its last exchange.  Two words
 // are used in turn, since a block may arrive at the next exchange before another has read this
@@ -25,6 +26,9 @@
 // see the mark and follow.  The words then hold arrivals that belong to no exchange, so a launch
 // that finds the mark leaves at its first exchange; fem_pic_status clears words and mark.
 #pragma once
+
+#include <cmath>
+#include <cstring>
 
 #include "internal.cuh"
 #ifdef __CUDACC__
@@ -41,6 +45,34 @@ constexpr uint64_t kGridStartNs = 30000000000ull, kGridWaitNs = 2000000000ull;
 // the sums that are added one by one (two copies of three doubles per block)
 constexpr size_t kGridLine = 128, kGridMark = 64;
 inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * blocks * 3 * 8; }
+
+// A sum's word: the exponent of its scale, a block's increment, and the total that the increments
+// of all blocks stand for (false: to be added one by one).
+constexpr int kWordExpect = 36;
+constexpr float kWordFits = 549755813888.f;              // 2^39
+constexpr long long kWordLeast = 1ll << 31;
+__host__ __device__ inline float word_pow2(int e) {
+    const uint32_t b = (uint32_t)(e + 127) << 23;
+    float f;
+    memcpy(&f, &b, 4);
+    return f;
+}
+// power of two that takes a total of about `expect` near 2^kWordExpect (0: no expectation)
+__host__ __device__ inline int word_exp(float expect) {
+    uint32_t b;
+    memcpy(&b, &expect, 4);
+    const int e = (int)((b >> 23) & 0xffu), s = kWordExpect - (e - 127);
+    return expect > 0.f && e > 0 && e < 255 ? (s < -96 ? -96 : s > 96 ? 96 : s) : 0;
+}
+__host__ __device__ inline unsigned long long word_put(float v, int e) {
+    const float x = v * word_pow2(e);
+    return (fabsf(x) < kWordFits ? (unsigned long long)llrintf(x) << 16 : 256ull) + 1ull;   // (a NaN does not fit)
+}
+__host__ __device__ inline bool word_total(unsigned long long d, int e, float* total) {
+    const long long t = (long long)d >> 16;
+    *total = (float)t * word_pow2(-e);
+    return ((d >> 8) & 255ull) == 0 && (t >= kWordLeast || t <= -kWordLeast);
+}
 
 #ifdef __CUDACC__
 
@@ -131,12 +163,6 @@ struct GridSync {
             }
         }
     }
-    // power of two that takes a total of about `expect` near 2^32 (0: no expectation)
-    static __device__ __forceinline__ int scale_exp(float expect) {
-        const int e = (int)((__float_as_uint(expect) >> 23) & 0xffu);
-        return expect > 0.f && e > 0 && e < 255 ? min(max(32 - (e - 127), -96), 96) : 0;
-    }
-    static __device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
 
     // grid barrier: what any thread wrote before is visible to every thread after
     __device__ __forceinline__ bool barrier() {
@@ -187,20 +213,14 @@ struct GridSync {
             int e[NV];
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                e[k] = scale_exp(expect[k]);
-                const float x = v[k] * pow2(e[k]);
-                const bool fits = fabsf(x) < 549755813888.f;   // 2^39, and finite
-                q[k] = (fits ? (unsigned long long)__float2ll_rn(x) << 16 : 256ull) + 1ull;
+                e[k] = word_exp(expect[k]);
+                q[k] = word_put(v[k], e[k]);
                 parts[k * nb + blockIdx.x] = v[k];             // for the sums added one by one
             }
             const bool ok = !sh->fail && arrive_wait<NV>(par, q, d);
             bool exact = false;
 #pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                const long long t = (long long)d[k] >> 16;
-                exact = exact || ((d[k] >> 8) & 255ull) != 0 || (t < 16777216ll && t > -16777216ll);
-                sh->tot[par][k] = __ll2float_rn(t) * pow2(-e[k]);
-            }
+            for (int k = 0; k < NV; ++k) exact = !word_total(d[k], e[k], &sh->tot[par][k]) || exact;
             if (!ok) abandon();
             sh->state[par] = ok ? (exact ? 2 : 0) : 1;
         }

@@ -19,4 +19,12 @@ int hs_met(double rr, double thr) { return solve_met(rr, thr) ? 1 : 0; }
 
 double hs_wait_seconds(int first) { return 1e-9 * (double)(first ? kGridStartNs : kGridWaitNs); }
 
+// the total of n blocks' partials as one grid exchange sums them; 0: the blocks add the floats instead
+int hs_word_sum(const float* v, int n, float expect, float* total) {
+    const int e = word_exp(expect);
+    unsigned long long d = 0;
+    for (int k = 0; k < n; ++k) d += word_put(v[k], e);
+    return (int)(d & 255ull) == n && word_total(d, e, total);
+}
+
 }  // extern "C"

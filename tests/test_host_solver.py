@@ -25,6 +25,7 @@ def hs(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(out)
     lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
+    lib.hs_word_sum.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_void_p]
     lib.hs_wait_seconds.restype = ctypes.c_double
     lib.hs_met.argtypes = [ctypes.c_double, ctypes.c_double]
     return lib
@@ -50,3 +51,40 @@ def test_first_exchange_waits_for_blocks_that_start_late(hs):
     to be there is many times the wait for blocks at work, and still bounded."""
     assert 2.0 <= hs.hs_wait_seconds(0) <= 5.0
     assert 10.0 * hs.hs_wait_seconds(0) <= hs.hs_wait_seconds(1) <= 60.0
+
+
+@pytest.mark.parametrize("blocks", [2, 152, 255])
+@pytest.mark.parametrize("kind", ["alike", "one_large", "signs"])
+def test_exchange_sums_are_as_fine_as_float_sums(hs, blocks, kind):
+    """The total that an exchange takes from its integer word is within 2^-23 of the exact one: half a
+    unit per block, at most 2^-24 of it, and its own rounding to a float.  Totals near their
+    expectation, and up to 16 times above or below, come from the word."""
+    rng = np.random.default_rng(blocks)
+    for log_ratio in range(-40, 16):
+        expect = np.float32(rng.uniform(1e-6, 1e-3))
+        total = float(expect) * 2.0 ** log_ratio
+        unit = 2.0 ** (np.frexp(expect)[1] - 1 - 36)      # of the word: the expectation's power of two is 2^36
+        if kind == "one_large":     # all the others rounded the same way, by nearly half a unit
+            v = np.full(blocks, 0.49 * unit)
+            v[0] = total
+        else:
+            v = rng.uniform(0.5, 1.5, blocks) * total / blocks
+            if kind == "signs":
+                v[1::2] *= -0.5
+        v = v.astype(np.float32)
+        got = np.zeros(1, np.float32)
+        used = hs.hs_word_sum(v.ctypes.data, blocks, expect, got.ctypes.data)
+        exact = float(v.astype(np.float64).sum())
+        if used:
+            assert abs(float(got[0]) - exact) <= 2.0 ** -23 * abs(exact), (log_ratio, got[0], exact)
+        assert used or abs(log_ratio) > 4 or (kind, blocks) != ("alike", 152)
+
+
+def test_exchange_sums_that_do_not_fit_are_left_to_the_floats(hs):
+    got = np.zeros(1, np.float32)
+    for bad in (NAN, INF, -INF, 1e30):
+        v = np.array([1.0, bad, 1.0], np.float32)
+        assert not hs.hs_word_sum(v.ctypes.data, 3, 1.0, got.ctypes.data)
+    for expect in (0.0, NAN, INF, -1.0, 1e-42):           # no expectation: units of one
+        v = np.full(3, 0.25, np.float32)
+        assert not hs.hs_word_sum(v.ctypes.data, 3, expect, got.ctypes.data)
