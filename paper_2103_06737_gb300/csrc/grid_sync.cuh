@@ -43,7 +43,8 @@ constexpr uint64_t kGridStartNs = 30000000000ull, kGridWaitNs = 2000000000ull;
 // device memory of one handle's exchanges (zeroed at setup): the words at rest and the mark of an
 // abandoned exchange, the words in use (two exchanges; a line each), then the blocks' partials for
 // the sums that are added one by one (two copies of three doubles per block)
-constexpr size_t kGridLine = 128, kGridMark = 64;
+constexpr size_t kGridLine = 128, kGridMark = 32;
+constexpr int kFail = 4;
 inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * blocks * 3 * 8; }
 
 // A sum's word: the exponent of its scale, a block's increment, and the total that the increments
@@ -80,8 +81,9 @@ struct GridSyncShared {
     double part64[3][32];
     float part[2][3][33];        // per-warp partials, by the exchange's parity
     float tot[2][2];
-    unsigned long long prev[2][2];   // what each word held after this block's last exchange on it
-    int fail;                    // the block does not arrive any more: its own wait ran out, or the mark is set
+    // [2 par + k]: what each word held after this block's last exchange on it; [kFail]: not 0, the
+    // block does not arrive any more (its own wait ran out, or the mark is set)
+    unsigned long long rest[5];
     int state[2];                // bit 0: a wait ran out, bit 1: add the partials one by one
 };
 
@@ -105,10 +107,10 @@ struct GridSync {
         lane = threadIdx.x & 31;
         wid = threadIdx.x >> 5;
         warps = blockDim.x >> 5;
-        // nothing changes the words at rest before every block's first arrival
-        if (!ONE && threadIdx.x < 4) s->prev[threadIdx.x >> 1][threadIdx.x & 1] =
+        // nothing changes the words at rest before every block's first arrival; the mark comes with them
+        if (!ONE && threadIdx.x < 5) s->rest[threadIdx.x] =
             *reinterpret_cast<volatile unsigned long long*>(mem + 8 * threadIdx.x);
-        if (threadIdx.x == 4) s->fail = ONE ? 0 : *mark();
+        if (ONE && threadIdx.x == 0) s->rest[kFail] = 0;
         __syncthreads();
     }
     __device__ __forceinline__ volatile int* mark() { return reinterpret_cast<volatile int*>(mem + kGridMark); }
@@ -121,7 +123,7 @@ struct GridSync {
     __device__ __forceinline__ void finish() {
         if constexpr (!ONE)
             for (int k = 0; k < 4; ++k)
-                *reinterpret_cast<volatile unsigned long long*>(mem + 8 * k) = sh->prev[k >> 1][k & 1];
+                *reinterpret_cast<volatile unsigned long long*>(mem + 8 * k) = sh->rest[k];
     }
     __device__ __forceinline__ unsigned long long* word(int par) {
         return reinterpret_cast<unsigned long long*>(mem + kGridLine * (1 + par));
@@ -149,12 +151,12 @@ struct GridSync {
             asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(c[0]) : "l"(w) : "memory");
 #pragma unroll
             for (int k = 0; k < NW; ++k) {
-                d[k] = c[k] - sh->prev[par][k];
+                d[k] = c[k] - sh->rest[2 * par + k];
                 all = all && (int)(d[k] & 255ull) == nb;
             }
             if (all) {
 #pragma unroll
-                for (int k = 0; k < NW; ++k) sh->prev[par][k] = c[k];
+                for (int k = 0; k < NW; ++k) sh->rest[2 * par + k] = c[k];
                 return true;
             }
             if ((spin & 1023u) == 1023u) {
@@ -175,7 +177,7 @@ struct GridSync {
         if (threadIdx.x == 0) {
             const unsigned long long q[1] = {1ull};
             unsigned long long d[1];
-            const bool ok = !sh->fail && arrive_wait<1>(par, q, d);
+            const bool ok = sh->rest[kFail] == 0 && arrive_wait<1>(par, q, d);
             if (!ok) abandon();
             sh->state[par] = ok ? 0 : 1;
         }
@@ -217,7 +219,7 @@ struct GridSync {
                 q[k] = word_put(v[k], e[k]);
                 parts[k * nb + blockIdx.x] = v[k];             // for the sums added one by one
             }
-            const bool ok = !sh->fail && arrive_wait<NV>(par, q, d);
+            const bool ok = sh->rest[kFail] == 0 && arrive_wait<NV>(par, q, d);
             bool exact = false;
 #pragma unroll
             for (int k = 0; k < NV; ++k) exact = !word_total(d[k], e[k], &sh->tot[par][k]) || exact;

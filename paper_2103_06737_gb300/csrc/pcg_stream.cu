@@ -114,7 +114,7 @@ struct Ring {
     const StreamArgs& a;
     unsigned char* buf;
     uint64_t *full, *empty;        // kStreamBars each
-    int* fail;                     // shared: a wait ran out, the block leaves at its next exchange
+    unsigned long long* fail;      // shared: a wait ran out, the block leaves at its next exchange
     uint64_t policy;
     int lane, warp, t0, nt;        // the block's tiles
     uint32_t count;                // items so far, over the whole launch: issued (producer) or used (consumer)
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_pcg_stream(StreamArgs a) 
         mbar_fence_init();
     }
     __syncthreads();
-    Ring R{a, dsm, full, empty, &shs.fail};
+    Ring R{a, dsm, full, empty, &shs.rest[kFail]};
     R.policy = evict_first_policy();
     R.lane = lane, R.warp = warp, R.t0 = t0, R.nt = nt;
     R.count = 0;
