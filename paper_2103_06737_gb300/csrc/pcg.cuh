@@ -27,6 +27,46 @@ namespace fempic {
 constexpr double kInnerMargin = 0.2;
 constexpr int kResMaxSlices = 96;   // slices of a block of the on-chip solver, at most
 
+// ---- records of the streamed solver (pcg_stream.cu)
+__host__ __device__ constexpr uint32_t align16(uint32_t b) { return (b + 15u) & ~15u; }
+constexpr int kConsumers = 15;            // consumer warps = slices of a tile; one more warp copies
+constexpr uint32_t kHeader = align16(8u * kConsumers);
+constexpr uint32_t kWide = 0x80000000u;   // meta flag: 32-bit columns
+
+enum { OP_F32, OP_LEARNED, OP_F64, OP_COUNT };
+// bytes of the parts of a record of w slots: bases, columns, values
+__host__ __device__ inline uint32_t base_bytes(uint32_t w, bool wide) { return wide ? 0u : align16(4u * w); }
+__host__ __device__ inline uint32_t col_bytes(uint32_t w, bool wide) { return wide ? 128u * w : 128u * ((w + 1u) / 2u); }
+__host__ __device__ inline uint32_t val_bytes(uint32_t w, int op) {
+    return op == OP_F32 ? 128u * w : op == OP_F64 ? 256u * w : 128u * ((w + 1u) / 2u);
+}
+__host__ __device__ inline uint32_t rec_bytes(uint32_t w, bool wide, int op) {
+    return w == 0 ? 0u : base_bytes(w, wide) + col_bytes(w, wide) + val_bytes(w, op);
+}
+// a tile's place in the ring
+inline uint32_t tile_bytes(uint32_t bytes) { return (bytes + 127u) & ~127u; }
+
+// The ring in shared memory.  A pass hides its copies behind its products only when two of its tiles
+// fit, and what the ring leaves free is L1 for the gathered vector (64^3 mesh: 51 us per iteration with
+// this much, 53 with all of it): as much as two FP64 tiles of the cube meshes' edge systems take
+// (19 slots a row, 2 x 93,568 bytes), more where the operator's own tiles are larger.
+constexpr size_t kStreamRing = 187392;
+
+// Rows of up to wmax slots as nseg records of at most seg slots each, alike in size: as few as let two
+// FP64 tiles fit in `room` bytes, whatever their column format (20 slots in the 230,656 bytes of
+// sm_103a).  Each more record costs a wait on the ring per slice.
+inline void stream_segments(int wmax, size_t room, int* nseg, int* seg) {
+    int most = 1;
+    auto two = [](int w) {
+        const uint32_t narrow = rec_bytes(w, false, OP_F64), wide = rec_bytes(w, true, OP_F64);
+        return (size_t)2 * tile_bytes(kHeader + kConsumers * (narrow > wide ? narrow : wide));
+    };
+    while (most < 0xffff && two(most + 1) <= room) ++most;
+    const int w = wmax > 1 ? wmax : 1;
+    *nseg = (w + most - 1) / most;
+    *seg = (w + *nseg - 1) / *nseg;
+}
+
 #ifdef __CUDACC__
 // FP64 scalars of a refinement, in shared memory: computed by one thread of each block from the
 // grid's sums.  With every thread computing them (two square roots and two quotients, 16 cycles of the

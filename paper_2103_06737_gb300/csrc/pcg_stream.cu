@@ -33,30 +33,9 @@
 namespace fempic {
 namespace {
 
-__host__ __device__ constexpr uint32_t align16(uint32_t b) { return (b + 15u) & ~15u; }
-#ifndef FP_STREAM_CONSUMERS
-#define FP_STREAM_CONSUMERS 15
-#endif
-#ifndef FP_STREAM_RING
-#define FP_STREAM_RING 187392
-#endif
-constexpr int kConsumers = FP_STREAM_CONSUMERS;      // consumer warps = slices of a tile; one more warp copies
 constexpr int kStreamThreads = 32 * (kConsumers + 1);
 constexpr int kStreamBars = 4;                       // tiles in flight, at most
-constexpr uint32_t kHeader = align16(8u * kConsumers);
 constexpr uint64_t kCopyWaitNs = 2000000000ull;
-constexpr uint32_t kWide = 0x80000000u;   // meta flag: 32-bit columns
-
-enum { OP_F32, OP_LEARNED, OP_F64, OP_COUNT };
-// bytes of the parts of a record of w slots: bases, columns, values
-__host__ __device__ __forceinline__ uint32_t base_bytes(uint32_t w, bool wide) { return wide ? 0u : align16(4u * w); }
-__host__ __device__ __forceinline__ uint32_t col_bytes(uint32_t w, bool wide) { return wide ? 128u * w : 128u * ((w + 1u) / 2u); }
-__host__ __device__ __forceinline__ uint32_t val_bytes(uint32_t w, int op) {
-    return op == OP_F32 ? 128u * w : op == OP_F64 ? 256u * w : 128u * ((w + 1u) / 2u);
-}
-__host__ __device__ __forceinline__ uint32_t rec_bytes(uint32_t w, bool wide, int op) {
-    return w == 0 ? 0u : base_bytes(w, wide) + col_bytes(w, wide) + val_bytes(w, op);
-}
 
 // rows that a pass reads once: past L1, whose room the gathered vector needs
 template <typename T>
@@ -726,7 +705,7 @@ static fp_status stream_layout(fem_pic* ctx, StreamPlan* P, int op, std::vector<
         return FP_EINVAL;
     }
     P->bytes[op] = off;
-    P->stage[op] = (int)((most + 127u) & ~127u);
+    P->stage[op] = (int)tile_bytes(most);
     FP_CUDA_TRY(ctx, cudaMalloc((void**)&P->rec[op], off + 128));
     FP_CUDA_TRY(ctx, cudaMemset(P->rec[op], 0, off + 128));   // headers of slices past the last: no slots
     FP_CUDA_TRY(ctx, cudaMalloc((void**)&P->meta[op], meta.size() * sizeof(uint2) + 16));
@@ -748,17 +727,18 @@ static fp_status stream_pack(fem_pic* ctx, StreamPlan* P, const Sell& S, const d
     return FP_OK;
 }
 
-// slots per record at most: two FP64 tiles of such records fit in the ring
-constexpr int kStreamSeg = 20;
-
 fp_status stream_setup(fem_pic* ctx, const Sell& S, const double* val, const float* val32, int64_t n, int wmax,
                        StreamPlan* P) {
     stream_free(P);
     P->n = n;
     P->ns = (int)((n + 31) / 32);
     P->nt = (P->ns + kConsumers - 1) / kConsumers;
-    P->nseg = std::max(1, (wmax + kStreamSeg - 1) / kStreamSeg);
-    P->seg = P->nseg > 1 ? kStreamSeg : std::max(1, wmax);
+    int optin = 0;
+    FP_CUDA_TRY(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    cudaFuncAttributes fa;
+    FP_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, (const void*)k_pcg_stream));
+    const size_t room = ((size_t)optin - fa.sharedSizeBytes) & ~(size_t)127;
+    stream_segments(wmax, room, &P->nseg, &P->seg);
     const size_t items = (size_t)P->ns * P->nseg;
     uint32_t* d = nullptr;
     FP_CUDA_TRY(ctx, cudaMalloc((void**)&d, items * 4 + 16));
@@ -773,14 +753,8 @@ fp_status stream_setup(fem_pic* ctx, const Sell& S, const double* val, const flo
     if (st == FP_OK) st = stream_layout(ctx, P, OP_F64, &where);
     if (st == FP_OK) st = stream_pack<OP_F64, double>(ctx, P, S, val, val, where);
     if (st != FP_OK) return st;
-    int optin = 0;
-    FP_CUDA_TRY(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-    cudaFuncAttributes fa;
-    FP_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, (const void*)k_pcg_stream));
-    const size_t room = (size_t)optin - fa.sharedSizeBytes;
     FP_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)k_pcg_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
-    P->ring = (int)std::min<size_t>(room, FP_STREAM_RING) & ~127;
-    if (P->ring < P->stage[OP_F64]) P->ring = (int)room & ~127;
+    P->ring = (int)std::min(room, std::max(kStreamRing, (size_t)2 * P->stage[OP_F64]));
     if (P->ring < P->stage[OP_F64]) {
         ctx->err = "fem_pic_field_setup: a tile does not fit in the streamed solver's ring";
         return FP_ECUDA;

@@ -2,6 +2,7 @@
 // tests/test_host_solver.py with g++.
 #include "../paper_2103_06737_gb300/csrc/field.cuh"
 #include "../paper_2103_06737_gb300/csrc/grid_sync.cuh"
+#include "../paper_2103_06737_gb300/csrc/pcg.cuh"
 
 using namespace fempic;
 
@@ -25,6 +26,15 @@ int hs_word_sum(const float* v, int n, float expect, float* total) {
     unsigned long long d = 0;
     for (int k = 0; k < n; ++k) d += word_put(v[k], e);
     return (int)(d & 255ull) == n && word_total(d, e, total);
+}
+
+// r: records per slice, their slots, bytes of an FP64 tile of full records with 16- and 32-bit columns
+void hs_segments(int wmax, int64_t room, int64_t* r) {
+    int nseg = 0, seg = 0;
+    stream_segments(wmax, (size_t)room, &nseg, &seg);
+    r[0] = nseg, r[1] = seg;
+    for (int wide = 0; wide < 2; ++wide)
+        r[2 + wide] = tile_bytes(kHeader + kConsumers * rec_bytes((uint32_t)seg, wide != 0, OP_F64));
 }
 
 }  // extern "C"

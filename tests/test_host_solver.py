@@ -25,6 +25,7 @@ def hs(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(out)
     lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
+    lib.hs_segments.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_void_p]
     lib.hs_word_sum.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_void_p]
     lib.hs_wait_seconds.restype = ctypes.c_double
     lib.hs_met.argtypes = [ctypes.c_double, ctypes.c_double]
@@ -88,3 +89,18 @@ def test_exchange_sums_that_do_not_fit_are_left_to_the_floats(hs):
     for expect in (0.0, NAN, INF, -1.0, 1e-42):           # no expectation: units of one
         v = np.full(3, 0.25, np.float32)
         assert not hs.hs_word_sum(v.ctypes.data, 3, expect, got.ctypes.data)
+
+
+def test_records_of_wide_rows_fit_twice(hs):
+    """However wide the rows, two FP64 tiles fit in the shared memory of an SM (227 KB less the kernel's
+    own 1,792 bytes), so that copies run beside products; rows of up to 20 slots (19 in the cube
+    meshes' edge systems) are one record; the records of a row are alike."""
+    room = 232448 - 1792
+    r = np.zeros(4, np.int64)
+    for wmax in [1, 2, 15, 18, 19, 20, 21, 22, 37, 38, 39, 57, 58, 64, 100, 1000, 1501, 30000]:
+        hs.hs_segments(wmax, room, r.ctypes.data)
+        nseg, seg, narrow, wide = (int(x) for x in r)
+        assert nseg * seg >= wmax > (nseg - 1) * seg
+        assert 2 * narrow <= room and 2 * wide <= room, wmax
+        assert nseg * seg - wmax < nseg
+        assert (nseg == 1) == (wmax <= 20)
