@@ -342,7 +342,8 @@ typedef struct {
  *   (Eq. wave_cont), A = M + dt^2/4 S (Newmark beta = 1/4), L = D0^T M D0 (the discrete
  *   Laplacian of Eq. discreteGauss).
  * PEC walls: edges and nodes on boundary faces are fixed at zero (their rows keep a unit
- * diagonal, their columns are removed).  Replaces any earlier setup.  Synchronous.
+ * diagonal, their columns are removed).  Replaces any earlier setup; one that fails leaves
+ * the handle without a field setup.  Synchronous.
  */
 fp_status fem_pic_field_setup(fem_pic_t* ctx, double dt, double eps, double mu);
 
@@ -542,6 +543,7 @@ fp_status fem_pic_learned_init(fem_pic_t* ctx, uint64_t seed, int sample_capacit
  *     mesh (fem_pic_learned_params) can be set on another of the same kind.
  */
 enum { FP_LEARNED_GUESS = 0, FP_LEARNED_PRECOND = 1 };
+/* Replaces the system's network; one that fails leaves the system without a network. */
 fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_capacity, int model);
 
 /* FP_LEARNED_PRECOND: the preconditioner's correction from the current weights, for the

@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <new>
 
 #include "async_copy.cuh"
 #include "field.cuh"
@@ -387,9 +388,10 @@ fp_status fill_info(fem_pic* ctx, int slot, double tol, fp_solve_info* info, cud
     info->fell_back = 0;
     if (ctx->field->learned_used[slot]) {
         int fl = 0;
-        FP_CUDA_TRY(ctx, cudaMemcpyAsync(&fl, learned_flag(ctx->field, ctx->field->slot_sys[slot]), sizeof(int),
-                                         cudaMemcpyDeviceToHost, s));
-        FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        if (const int* flag = learned_flag(ctx->field, ctx->field->slot_sys[slot])) {   // null: no network any more
+            FP_CUDA_TRY(ctx, cudaMemcpyAsync(&fl, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+            FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        }
         info->precond = FP_PC_LEARNED;
         info->fell_back = fl;
     }
@@ -571,18 +573,7 @@ void field_free(fem_pic* ctx) {
 
 using namespace fempic;
 
-extern "C" {
-
-fp_status fem_pic_field_setup(fem_pic_t* ctx, double dt, double eps, double mu) {
-    return fem_pic_field_setup_bc(ctx, dt, eps, mu, FP_BC_PEC);
-}
-
-fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double mu, int bc) {
-    if (!ctx || !(dt > 0.0) || !(eps > 0.0) || !(mu > 0.0) || (bc != FP_BC_PEC && bc != FP_BC_NEUMANN)) {
-        if (ctx) ctx->err = "fem_pic_field_setup: dt, eps and mu must be positive, bc FP_BC_PEC or FP_BC_NEUMANN";
-        return FP_EINVAL;
-    }
-    field_free(ctx);
+static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, int bc) {
     FieldDev* F = new FieldDev();
     ctx->field = F;
     const HostComplex& hc = ctx->hc;
@@ -887,6 +878,32 @@ fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double m
         for (double v : a) F->alpha_sum += v;
         if (st == FP_OK) st = up(ctx, &F->alpha, a);
         if (st == FP_OK) FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->msum, kMeanBlocks * sizeof(double)));
+    }
+    return st;
+}
+
+extern "C" {
+
+fp_status fem_pic_field_setup(fem_pic_t* ctx, double dt, double eps, double mu) {
+    return fem_pic_field_setup_bc(ctx, dt, eps, mu, FP_BC_PEC);
+}
+
+fp_status fem_pic_field_setup_bc(fem_pic_t* ctx, double dt, double eps, double mu, int bc) {
+    if (!ctx || !(dt > 0.0) || !(eps > 0.0) || !(mu > 0.0) || (bc != FP_BC_PEC && bc != FP_BC_NEUMANN)) {
+        if (ctx) ctx->err = "fem_pic_field_setup: dt, eps and mu must be positive, bc FP_BC_PEC or FP_BC_NEUMANN";
+        return FP_EINVAL;
+    }
+    field_free(ctx);
+    fp_status st;
+    try {
+        st = field_setup(ctx, dt, eps, mu, bc);
+    } catch (const std::bad_alloc&) {   // no exception crosses the C ABI
+        ctx->err = "fem_pic_field_setup: out of host memory";
+        st = FP_EINVAL;
+    }
+    if (st != FP_OK) {   // nothing half-built: the handle is as before its first field setup
+        field_free(ctx);
+        (void)cudaGetLastError();
     }
     return st;
 }

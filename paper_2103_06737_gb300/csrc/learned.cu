@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <random>
 #include <vector>
 
@@ -1008,14 +1009,9 @@ fp_status fem_pic_learned_init(fem_pic_t* ctx, uint64_t seed, int sample_capacit
     return fem_pic_learned_init_model(ctx, seed, sample_capacity, FP_LEARNED_GUESS);
 }
 
-fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_capacity, int model) {
-    if (!ctx || !ctx->field || sample_capacity < 0 || (model != FP_LEARNED_GUESS && model != FP_LEARNED_PRECOND)) {
-        if (ctx) ctx->err = "fem_pic_learned_init: bad model or capacity (or fem_pic_field_setup not called)";
-        return FP_EINVAL;
-    }
+static fp_status learned_setup(fem_pic_t* ctx, uint64_t seed, int sample_capacity, int model) {
     FieldDev* F = ctx->field;
     const int sys = F->learned_sys;
-    learned_free(F, sys);
     LearnedDev* L = new LearnedDev();
     F->learned[sys] = L;
     const HostFields& H = F->host;
@@ -1163,6 +1159,27 @@ fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_c
     FP_CUDA_TRY(ctx, cudaMemset(L->flag, 0, sizeof(int)));
     FP_CUDA_TRY(ctx, cudaDeviceSynchronize());
     return FP_OK;
+}
+
+fp_status fem_pic_learned_init_model(fem_pic_t* ctx, uint64_t seed, int sample_capacity, int model) {
+    if (!ctx || !ctx->field || sample_capacity < 0 || (model != FP_LEARNED_GUESS && model != FP_LEARNED_PRECOND)) {
+        if (ctx) ctx->err = "fem_pic_learned_init: bad model or capacity (or fem_pic_field_setup not called)";
+        return FP_EINVAL;
+    }
+    FieldDev* F = ctx->field;
+    learned_free(F, F->learned_sys);
+    fp_status st;
+    try {
+        st = learned_setup(ctx, seed, sample_capacity, model);
+    } catch (const std::bad_alloc&) {   // no exception crosses the C ABI
+        ctx->err = "fem_pic_learned_init: out of host memory";
+        st = FP_EINVAL;
+    }
+    if (st != FP_OK) {   // nothing half-built: the system has no network
+        learned_free(F, F->learned_sys);
+        (void)cudaGetLastError();
+    }
+    return st;
 }
 
 fp_status fem_pic_learned_mode(fem_pic_t* ctx, int collect, int active) {

@@ -769,11 +769,23 @@ fp_status stream_setup(fem_pic* ctx, const Sell& S, const double* val, const flo
 fp_status stream_learned_room(fem_pic* ctx, StreamPlan* P) {
     if (!P->on || P->rec[OP_LEARNED]) return FP_OK;
     std::vector<PackItem> where;
-    const fp_status st = stream_layout(ctx, P, OP_LEARNED, &where);
-    if (st != FP_OK) return st;
-    FP_CUDA_TRY(ctx, cudaMalloc(&P->where, where.size() * sizeof(PackItem) + 16));
-    FP_CUDA_TRY(ctx, cudaMemcpy(P->where, where.data(), where.size() * sizeof(PackItem), cudaMemcpyHostToDevice));
-    return FP_OK;
+    fp_status st = stream_layout(ctx, P, OP_LEARNED, &where);
+    if (st == FP_OK) {
+        const size_t bytes = where.size() * sizeof(PackItem);
+        cudaError_t e = cudaMalloc(&P->where, bytes + 16);
+        if (e == cudaSuccess) e = cudaMemcpy(P->where, where.data(), bytes, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            ctx->err = std::string("fem_pic_learned_init: the streamed solver's records: ") + cudaGetErrorString(e);
+            st = FP_ECUDA;
+        }
+    }
+    if (st != FP_OK) {   // all of it or nothing: the packing takes records for complete
+        cudaFree(P->rec[OP_LEARNED]);
+        cudaFree(P->meta[OP_LEARNED]);
+        cudaFree(P->where);
+        P->rec[OP_LEARNED] = nullptr, P->meta[OP_LEARNED] = nullptr, P->where = nullptr;
+    }
+    return st;
 }
 
 fp_status stream_learned_pack(fem_pic* ctx, StreamPlan* P, const Sell& S, const double* val, const __nv_bfloat16* pre,

@@ -74,3 +74,25 @@ def test_abandoned_exchange_is_reported_and_reset(n):
     assert (again["iters"], again["outer"], again["rel_res"]) == (info["iters"], info["outer"], info["rel_res"])
     assert lib.status() == F.FP_OK
     lib.close()
+
+
+@pytest.mark.parametrize("model", [F.FP_LEARNED_GUESS, F.FP_LEARNED_PRECOND])
+def test_failed_learned_init_leaves_no_network(model):
+    """A network whose sample store does not fit on any device: the system is left without one, so
+    that a step that asks for it is refused, and everything else works on."""
+    lib = _lib(9)
+    with pytest.raises(F.FemPicError):
+        F.fem_pic_learned_init_model(lib.h, seed=1, sample_capacity=2**31 - 1, model=model)
+    E = [torch.zeros(lib.n_edges, dtype=torch.float64, device="cuda") for _ in range(3)]
+    Q = torch.zeros(lib.n_nodes, dtype=torch.float32, device="cuda")
+    step = lambda pc: F.fem_pic_field_step(lib.h, E[0], E[1], E[2], None, None, None, Q, tol=1e-10, precond=pc)
+    with pytest.raises(F.FemPicError, match="learned_init"):
+        step(F.FP_PC_LEARNED)
+    with pytest.raises(F.FemPicError):
+        F.fem_pic_learned_params(lib.h)
+    assert step(F.FP_PC_JACOBI)[0] == F.FP_OK
+    F.fem_pic_learned_init_model(lib.h, seed=1, sample_capacity=1, model=model)
+    if model == F.FP_LEARNED_PRECOND:
+        F.fem_pic_learned_build(lib.h)
+    assert step(F.FP_PC_LEARNED)[0] == F.FP_OK and lib.status() == F.FP_OK
+    lib.close()
