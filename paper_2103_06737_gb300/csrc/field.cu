@@ -557,11 +557,11 @@ void field_free(fem_pic* ctx) {
     FieldDev* F = ctx->field;
     if (!F) return;
     learned_free(F);
-    void* ptrs[] = {F->e_rp, F->e_col, F->n_rp, F->n_col, F->Mv, F->Sv, F->Av, F->Adinv, F->Lv, F->Ldinv,
+    void* ptrs[] = {F->e_rp, F->e_col, F->n_rp, F->n_col, F->Adinv, F->Ldinv,
                     F->edge_fixed, F->node_fixed, F->face_edges, F->r, F->z, F->p, F->q, F->rhs, F->tmp,
-                    F->delta, F->qd, F->red, F->out, F->Av32, F->Adinv32, F->Lv32, F->Ldinv32, F->r32,
+                    F->delta, F->qd, F->red, F->out, F->Ldinv32, F->r32,
                     F->z32, F->p32, F->q32, F->c32, F->s32, F->d32[0], F->d32[1], F->se_d16, F->sn_d16, F->pe_ptr, F->pe_w, F->pe_col, F->perm_e, F->pe_A, F->pe_A32, F->pe_dinv32, F->pb, F->px, F->alpha, F->msum, F->se_ptr, F->se_w, F->se_col, F->sn_ptr, F->sn_w,
-                    F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->se_A32, F->sn_L32, F->sync, F->res[0].pp, F->res[1].pp};
+                    F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->sn_L32, F->sync, F->res[0].pp, F->res[1].pp};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (StreamPlan& P : F->stream) stream_free(&P);
@@ -608,21 +608,13 @@ static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, i
     if (st == FP_OK) st = up(ctx, &F->e_col, H.e_col);
     if (st == FP_OK) st = up(ctx, &F->n_rp, H.n_rp);
     if (st == FP_OK) st = up(ctx, &F->n_col, H.n_col);
-    if (st == FP_OK) st = up(ctx, &F->Mv, H.M);
-    if (st == FP_OK) st = up(ctx, &F->Sv, H.S);
-    if (st == FP_OK) st = up(ctx, &F->Av, A);
     if (st == FP_OK) st = up(ctx, &F->Adinv, Ad);
-    if (st == FP_OK) st = up(ctx, &F->Lv, H.L);
     if (st == FP_OK) st = up(ctx, &F->Ldinv, Ld);
     if (st == FP_OK) st = up(ctx, &F->edge_fixed, H.edge_fixed);
     if (st == FP_OK) st = up(ctx, &F->node_fixed, H.node_fixed);
     if (st == FP_OK) st = up(ctx, &F->face_edges, fe);
     {
-        std::vector<float> a32(A.begin(), A.end()), ad32(Ad.begin(), Ad.end()), l32(H.L.begin(), H.L.end()),
-            ld32(Ld.begin(), Ld.end());
-        if (st == FP_OK) st = up(ctx, &F->Av32, a32);
-        if (st == FP_OK) st = up(ctx, &F->Adinv32, ad32);
-        if (st == FP_OK) st = up(ctx, &F->Lv32, l32);
+        std::vector<float> ld32(Ld.begin(), Ld.end());
         if (st == FP_OK) st = up(ctx, &F->Ldinv32, ld32);
     }
     {
@@ -684,14 +676,12 @@ static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, i
         };
         sell(H.e_rp, H.e_col, hc.ne, &ptr, &w, &scol, &map);
         std::vector<double> sM = gather(map, H.M), sS = gather(map, H.S), sA = gather(map, A);
-        std::vector<float> sA32(sA.begin(), sA.end());
         if (st == FP_OK) st = up(ctx, &F->se_ptr, ptr);
         if (st == FP_OK) st = up(ctx, &F->se_w, w);
         if (st == FP_OK) st = up(ctx, &F->se_col, scol);
         if (st == FP_OK) st = up(ctx, &F->se_M, sM);
         if (st == FP_OK) st = up(ctx, &F->se_S, sS);
         if (st == FP_OK) st = up(ctx, &F->se_A, sA);
-        if (st == FP_OK) st = up(ctx, &F->se_A32, sA32);
         {
             // Row order of the mixed solver's Newmark operator.  Edge ids are lexicographic in
             // (i, j), so the edges leaving a node are consecutive and a 32-row slice mixes edges
@@ -794,7 +784,6 @@ static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, i
             if (st == FP_OK) st = up(ctx, &F->pe_A, pA);
             if (st == FP_OK) st = up(ctx, &F->pe_A32, pA32);
             if (st == FP_OK) st = up(ctx, &F->pe_dinv32, pdinv);
-            if (st == FP_OK) FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->pb, ne * sizeof(double)));
             if (st == FP_OK) FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->px, ne * sizeof(double)));
         }
         sell(H.n_rp, H.n_col, hc.nn, &ptr, &w, &scol, &map);
@@ -860,6 +849,13 @@ static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, i
         const int wmax = F->hwidth[sys].empty() ? 0 : *std::max_element(F->hwidth[sys].begin(), F->hwidth[sys].end());
         st = stream_setup(ctx, nm ? Sell{F->pe_ptr, F->pe_w, F->pe_col} : Sell{F->sn_ptr, F->sn_w, F->sn_col},
                           nm ? F->pe_A : F->sn_L, nm ? F->pe_A32 : F->sn_L32, nm ? hc.ne : hc.nn, wmax, &F->stream[sys]);
+        if (st == FP_OK && nm) FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->pb, hc.ne * sizeof(double)));
+        if (F->res[sys].on) continue;
+        // only the on-chip solver reads the unpacked FP32 operator and its 16-bit offsets
+        cudaFree(nm ? F->pe_A32 : F->sn_L32);
+        cudaFree(nm ? F->se_d16 : F->sn_d16);
+        (nm ? F->pe_A32 : F->sn_L32) = nullptr;
+        (nm ? F->se_d16 : F->sn_d16) = nullptr;
     }
     if (st == FP_OK) {
         FP_CUDA_TRY(ctx, cudaMalloc(&F->sync, grid_sync_bytes(ctx->sm_count)));

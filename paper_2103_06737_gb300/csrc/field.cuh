@@ -76,28 +76,27 @@ struct FieldDev {
     int64_t ne = 0, nn = 0, nf = 0;
     HostFields host;
     int32_t *e_rp = nullptr, *e_col = nullptr, *n_rp = nullptr, *n_col = nullptr;
-    double *Mv = nullptr, *Sv = nullptr, *Av = nullptr, *Adinv = nullptr, *Lv = nullptr, *Ldinv = nullptr;
+    double *Adinv = nullptr, *Ldinv = nullptr;
     uint8_t *edge_fixed = nullptr, *node_fixed = nullptr;
     int32_t* face_edges = nullptr;  // [3 nf]: (i,j), (j,k), (i,k) of face (i<j<k)
     double *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *rhs = nullptr, *tmp = nullptr,
            *delta = nullptr, *qd = nullptr;
-    float *Av32 = nullptr, *Adinv32 = nullptr, *Lv32 = nullptr, *Ldinv32 = nullptr;  // FP32 copies
+    float* Ldinv32 = nullptr;       // FP32 copy
     // sliced ELLPACK (slices of 32 rows, column-major inside a slice): coalesced loads of the
     // values and columns of 32 consecutive rows
     int32_t *se_ptr = nullptr, *se_w = nullptr, *se_col = nullptr, *sn_ptr = nullptr, *sn_w = nullptr,
             *sn_col = nullptr;
     double *se_M = nullptr, *se_S = nullptr, *se_A = nullptr, *sn_L = nullptr;
-    float *se_A32 = nullptr, *sn_L32 = nullptr;
+    float* sn_L32 = nullptr;        // FP32 copy, where the on-chip solver runs
     float *r32 = nullptr, *z32 = nullptr, *p32 = nullptr, *q32 = nullptr, *c32 = nullptr;
     float *s32 = nullptr, *d32[2] = {nullptr, nullptr};  // Chebyshev preconditioner scratch
     double lmax[2] = {2.0, 2.0};    // estimated largest eigenvalue of D^-1 A, Newmark and Gauss systems
-    // column offsets col - row as int16 in the SELL layout, for the on-chip solver (null when some
-    // offset does not fit)
+    // column offsets col - row as int16 in the SELL layout, for the on-chip solver (null without it)
     int16_t *se_d16 = nullptr, *sn_d16 = nullptr;
     // The mixed solver's copy of the Newmark operator in its own row order: solver row r is
-    // edge perm_e[r] (rows and columns renumbered alike).  Right-hand side and guess are
-    // gathered into pb / px before each solve and the solution scattered back after it.
-    // se_d16 and hwidth of the Newmark system describe this copy.
+    // edge perm_e[r] (rows and columns renumbered alike).  A solve holds its solution in px in
+    // this order, the streamed solver its right-hand side in pb (null without it); pe_A32 is null
+    // without the on-chip solver.  se_d16 and hwidth of the Newmark system describe this copy.
     int32_t *pe_ptr = nullptr, *pe_w = nullptr, *pe_col = nullptr, *perm_e = nullptr;
     double* pe_A = nullptr;
     float *pe_A32 = nullptr, *pe_dinv32 = nullptr;
