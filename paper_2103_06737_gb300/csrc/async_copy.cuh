@@ -63,12 +63,6 @@ __device__ __forceinline__ void bulk_wait_read_all() {
 // waits until every committed bulk group has completed (its writes performed)
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// asks the TMA engine to bring a global range into L2 (no completion to wait for); src 16-byte
-// aligned, bytes a multiple of 16
-__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(

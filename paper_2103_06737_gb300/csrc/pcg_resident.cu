@@ -31,8 +31,9 @@
 namespace fempic {
 namespace {
 
-// the two signed 16-bit column offsets of a slot pair, kept in 32-bit registers throughout (a
-// build that let them live in 16-bit registers spilled those and read out of range)
+// The two signed 16-bit column offsets of a slot pair, in 32-bit registers throughout.  Earlier builds
+// that held them in 16-bit registers, and spilled those, read out of range; the spill is the
+// suspected cause, not a proven one.  Every offset is range-checked where it enters shared memory.
 __device__ __forceinline__ int offset_lo(int d) {
     int o;
     asm("bfe.s32 %0, %1, 0, 16;" : "=r"(o) : "r"(d));
@@ -97,12 +98,9 @@ struct LearnedValues {  // the learned correction's slots, from global memory (S
 // per-row vectors of a block in shared memory, in this order (the last two for the polynomial only)
 enum { RV_R, RV_Z, RV_P, RV_Q, RV_C, RV_DI, RV_JACOBI, RV_S = RV_JACOBI, RV_D, RV_COUNT };
 
-#ifndef FP_RES_PC
-#define FP_RES_PC 4
-#endif
 template <int THREADS, bool ONE>
 struct Resident {
-    static constexpr int PC = THREADS <= 512 ? 8 : FP_RES_PC;   // slot pairs of a row in flight
+    static constexpr int PC = THREADS <= 512 ? 8 : 4;   // slot pairs of a row in flight
     const ResidentArgs& a;
     GridSync<ONE>& g;
     int lane, warp, W, s0, nsl, rows_pb;
@@ -387,11 +385,9 @@ void* resident_kernel(int threads, bool one) {
 
 }  // namespace
 
-// A block takes at least FP_RES_MIN_SLICES slices (fewer blocks for small systems: each exchange
-// then has fewer words to wait for).
-#ifndef FP_RES_MIN_SLICES
-#define FP_RES_MIN_SLICES 4
-#endif
+// A block takes at least this many slices (fewer blocks for small systems: each exchange then has
+// fewer words to wait for).
+constexpr int kResMinSlices = 4;
 fp_status resident_setup(fem_pic* ctx, int64_t n, const std::vector<int32_t>& width, ResidentPlan* P) {
     *P = ResidentPlan();
     const int64_t ns = (int64_t)width.size();
@@ -399,7 +395,7 @@ fp_status resident_setup(fem_pic* ctx, int64_t n, const std::vector<int32_t>& wi
     std::vector<int32_t> pp(ns + 1, 0);
     for (int64_t s = 0; s < ns; ++s) pp[s + 1] = pp[s] + (width[s] + 1) / 2;
     const bool one = n <= 1024;
-    const int64_t nb0 = one ? 1 : std::min<int64_t>(std::min(ctx->sm_count, 255), (ns + FP_RES_MIN_SLICES - 1) / FP_RES_MIN_SLICES);
+    const int64_t nb0 = one ? 1 : std::min<int64_t>(std::min(ctx->sm_count, 255), (ns + kResMinSlices - 1) / kResMinSlices);
     const int64_t spb = (ns + nb0 - 1) / nb0;
     if (spb > kResMaxSlices) return FP_OK;
     const int64_t warps = one ? 20 : kResThreads / 32, rounds = (spb + warps - 1) / warps;   // slices per warp

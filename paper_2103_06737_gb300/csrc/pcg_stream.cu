@@ -1,9 +1,10 @@
 // Mixed-precision field solve whose operator is streamed from HBM (or L2) once per product.
 //
 // The method is pcg.cuh's, here for systems whose FP32 operator does not fit in the SMs' shared
-// memory (the edge system from about 40^3, the node system from about 66^3).  A product reads its
-// operator once, so it is bound by the operator's bytes and, behind them, by the latency of the
-// chain column -> gathered entry.  So here
+// memory (cube meshes on 152 SMs: the edge system from 34^3, 33^3 with the polynomial's two more
+// vectors; the node system from about 66^3, 64^3 with them).  A product reads its operator once,
+// so it is bound by the operator's bytes and, behind them, by the latency of the chain
+// column -> gathered entry.  So here
 //  - the operator is packed into one record per 32-row slice: per slot a 32-bit base column, per
 //    entry a 16-bit column offset (relative to base + lane) and the value: 6.1 bytes per FP32
 //    entry instead of 8 (the learned correction 4.1 instead of 6, the FP64 operator 10.1
