@@ -112,6 +112,9 @@ def parse():
     ap.add_argument("--drift-tol", type=float, default=1e-6,
                     help="second run of the Gauss-law comparison with this solver tolerance for the two "
                          "unprojected systems (the projected step keeps --tol; 0: skip)")
+    ap.add_argument("--detail", default="",
+                    help="file for the whole record as JSON (every measurement of the run); the printed line is its "
+                         "headline")
     ap.add_argument("--min-warmup-s", type=float, default=1.5,
                     help="keep warming up at least this long (clock sampling under load)")
     return ap.parse_args()
@@ -1661,6 +1664,53 @@ def run_also(args):
     return res
 
 
+LINE_BYTES = 2900   # of the printed line: longer ones (the whole record is 20 KB) were cut by what reads them
+
+
+def _pick(d, *keys):
+    return None if d is None else {k: d[k] for k in keys if k in d}
+
+
+def _short(x):
+    """x with its numbers to seven digits (whole numbers stay whole)."""
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v) for v in x]
+    return float(f"{x:.7g}") if isinstance(x, float) else x
+
+
+def headline(out, limit=LINE_BYTES):
+    """The printed line: what the record's headline metric needs, then as much of the rest as fits."""
+    line = _pick(out, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "gpu_launches", "status", "clocks")
+    line["config"] = _pick(out["config"], "workload", "mesh", "particles", "alive_in_timed_steps", "species", "n_tets",
+                           "n_edges", "dt_s", "sort_every", "precision", "l2", "parallelism", "step")
+    line["e2e"] = _pick(out.get("e2e"), "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step")
+    roof = ("kernel", "bound", "achieved", "peak", "peak_kind", "unit", "frac", "avg_launch_ms", "iterations_per_launch",
+            "traffic")
+    fs = out.get("field_solve") or {}
+    learned = fs.get("learned_vs_plain") or {}
+    rest = [
+        ("cpu_baseline", _pick(out.get("cpu_baseline"), "value", "unit", "cores", "kind", "sample")),
+        ("config", {**line["config"], "deposits": out["config"].get("deposits")}),
+        ("field_solve", fs and {**_pick(fs, "ms_per_step", "ms_newmark_cg", "ms_gauss_cg", "newmark_iters_mean",
+                                       "gauss_iters_mean", "max_rel_res", "precond"),
+                               "learned_vs_plain_ms": {k: v["learned_vs_plain_ms"] for k, v in learned.items()
+                                                       if isinstance(v, dict) and "learned_vs_plain_ms" in v}}),
+        ("roofline", _pick(out.get("roofline"), *roof)),
+        ("workloads", {k: _pick(v, "value", "ms_per_step") for k, v in (out.get("workloads") or {}).items()} or None),
+        ("roofline_push", _pick(out.get("roofline_push"), *roof)),
+        ("residuals", _pick((out.get("residuals") or {}).get("per_step"), "continuity_interior_rel_max", "divB_rel_max")),
+        ("adams", _pick(out.get("adams"), "particle_steps_per_s", "ms_per_call")),
+        ("fp64_mode", _pick(out.get("fp64_mode"), "particle_steps_per_s", "ms_per_call")),
+    ]
+    for k, v in rest:
+        if v and len(json.dumps(_short({**line, k: v}))) <= limit:
+            line[k] = v
+    return _short(line)
+
+
 def main():
     args = parse()
     if args.impl == "reference":
@@ -1674,7 +1724,10 @@ def main():
             out["workloads"] = also
         if world == 1 and not args.no_cpu_baseline:
             out["cpu_baseline"] = cpu_baseline(args, wl, args.cpu_seconds)
-        print(json.dumps(out), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(out, f)
+        print(json.dumps(headline(out)), flush=True)
 
 
 if __name__ == "__main__":
