@@ -251,9 +251,6 @@ def push_call_bytes(n_particles, n_tets):
     return 56 * n_particles + 230 * n_tets
 
 
-L2_BYTES = 129e6
-
-
 def pcg_bytes_per_iter(n_rows, nnz, val_bytes=8):
     """Minimal DRAM bytes of one FP64 Jacobi-PCG iteration (two barriers per iteration): the
     operator once (value + column index per nonzero) and 13 passes over n-vectors
@@ -277,6 +274,27 @@ def mixed_solve_bytes(n_rows, nnz, inner_iters, outer, deg=1):
     start = outer * (prec + op + (8 + 4 + 4 * 4) * n_rows + (8 + 8 + 4) * n_rows)
     resid = (outer + 1) * (nnz * 10.125 + (8 + 8 + 8 + 4) * n_rows)
     return inner + start + resid
+
+
+SMEM_SOLVER_BYTES = 152 * 230e3   # shared memory of the SMs that one block each of a solver can use
+
+
+def mixed_kernel(n_rows, nnz, deg=1):
+    """Which mixed solver a system runs in: on chip where its FP32 operator (4 B value + 2 B column
+    offset per nonzero) and six FP32 vectors, eight with a polynomial, fit in the SMs' shared memory
+    with a tenth to spare for padding and uneven shares (the library decides by the shares themselves;
+    the rule may differ from it for cube meshes of 32^3 to 34^3, edge system, and 62^3 to 66^3, node
+    system)."""
+    held = 6 * nnz + 4 * (8 if deg > 1 else 6) * n_rows
+    return "k_pcg_resident" if held <= 0.9 * SMEM_SOLVER_BYTES else "k_pcg_stream"
+
+
+def resident_solve_bytes(n_rows, nnz, outer):
+    """Bytes one on-chip mixed solve moves: the FP32 operator and D^-1 into shared memory once; per
+    refinement the FP64 operator (12 B per nonzero), x read and written, r64 written and read; the
+    right-hand side and its residual at the start, the solution at the end.  Inner iterations read
+    gathered vector entries only, through L2."""
+    return nnz * 6 + 4 * n_rows + outer * (12 * nnz + 32 * n_rows) + 32 * n_rows
 
 
 def measured_traffic(kernel: str, workload: str, iterations=None):
@@ -1278,17 +1296,18 @@ def run_gpu(args):
                     # solve's (inner) CG iterations
                     byt = cg_iter_bytes(rows, nz) * max(its, 1)
                     lrn = bool(main_pc & (F.FP_PC_LEARNED if k_sys == 0 else F.FP_PC_LEARNED_GAUSS))
-                    model = (mixed_solve_bytes(rows, nz, its, outs, 1 if lrn else main_pdeg[k_sys]) if mixed else
-                             pcg_bytes_per_iter(rows, nz) * max(its, 1))
-                    if lrn:   # one product with the BF16 learned correction per inner iteration
+                    deg = 1 if lrn else main_pdeg[k_sys]
+                    kern = mixed_kernel(rows, nz, deg) if mixed else "k_pcg"
+                    on_chip = kern == "k_pcg_resident"
+                    model = (pcg_bytes_per_iter(rows, nz) * max(its, 1) if not mixed else
+                             resident_solve_bytes(rows, nz, outs) if on_chip else
+                             mixed_solve_bytes(rows, nz, its, outs, deg))
+                    if lrn and not on_chip:   # one product with the BF16 learned correction per inner iteration
                         model += its * nz * 4.125
-                    op_bytes = nz * 6.125 * 1.2      # FP32 SELL operator (value + packed column), ~1.2x padding
-                    on_chip = op_bytes < L2_BYTES
-                    traffic = measured_traffic(("k_pcg_stream/" if mixed else "k_pcg/") + ph +
-                                               ("/learned" if lrn else ""), wl.name, its)
+                    traffic = measured_traffic(kern + "/" + ph + ("/learned" if lrn else ""), wl.name, its)
                     pc_name = ("learned preconditioner" if lrn else
                                f"Chebyshev-Jacobi degree {main_pdeg[k_sys]}" if main_pdeg[k_sys] > 1 else "Jacobi")
-                    name = ("k_pcg_resident or k_pcg_stream (" + ph.split("_")[1] + f" system, FP32 inner PCG, {pc_name}, FP64 residual)"
+                    name = (f"{kern} (" + ph.split("_")[1] + f" system, FP32 inner PCG, {pc_name}, FP64 residual)"
                             if mixed else "k_pcg (" + ph.split("_")[1] + " system, FP64)")
                     ach = byt / (avg * 1e-3) / 1e9
                     cand.append((avg, {
@@ -1303,16 +1322,16 @@ def run_gpu(args):
                         "rows": rows, "nnz": nz,
                         "model_bytes_per_launch": model,
                         "model_frac": model / (avg * 1e-3) / 1e9 / peak,
-                        "model_rule": ("what the mixed solver moves: the FP32 operator (6.1 B per nonzero) once per "
-                                       "product, deg products per inner iteration, FP32 vector passes, FP64 "
-                                       "residuals per refinement" if mixed else "FP64 PCG, 12 B per nonzero + "
-                                       "13 FP64 vector passes per iteration"),
+                        "model_rule": ("FP64 PCG, 12 B per nonzero + 13 FP64 vector passes per iteration" if not mixed
+                                       else "the FP32 operator once per solve, the FP64 operator and FP64 vectors per "
+                                       "refinement" if on_chip else "the FP32 operator (6.1 B per nonzero) once per "
+                                       "product, deg products per inner iteration, FP32 vector passes, FP64 residuals "
+                                       "per refinement"),
                         "traffic": traffic,
                         "traffic_frac": None if traffic is None else traffic / (avg * 1e-3) / 1e9 / peak,
-                        "note": ("the FP32 operator fits on chip (shared memory / L2): DRAM traffic is about one "
-                                 "read of it per launch and the kernel is bound by its grid barriers and gather "
+                        "note": ("operator and vectors in shared memory: bound by the grid exchanges and the gathers' "
                                  "latency, not by HBM" if on_chip else
-                                 "the FP32 operator is larger than L2: every product streams it from HBM")}))
+                                 "every product streams the operator from HBM, or from L2 where it stays there")}))
             cand.append((fast_avg, roof_push))
             roof = max(cand, key=lambda c: c[0])[1]
         out = {

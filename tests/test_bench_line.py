@@ -66,3 +66,16 @@ def test_line_without_the_optional_measurements():
     del out["workloads"], out["cpu_baseline"]
     d = json.loads(json.dumps(bench.headline(out)))
     assert d["e2e"] is None and "field_solve" not in d and "adams" not in d and d["value"] > 0
+
+
+def test_mixed_kernel_names_the_solver_that_runs():
+    """Rows and entries of the cube meshes' systems (nnz about 15.5 per edge row and 13 per node row with
+    PEC walls): what the sizes measured with the library showed."""
+    edges = lambda n: 7 * n ** 3 + 9 * n ** 2 + 3 * n
+    nodes = lambda n: (n + 1) ** 3
+    for n, kern in ((4, "k_pcg_resident"), (32, "k_pcg_resident"), (36, "k_pcg_stream"), (64, "k_pcg_stream"),
+                    (96, "k_pcg_stream")):
+        for deg in (1, 3):
+            assert bench.mixed_kernel(edges(n), int(15.5 * edges(n)), deg) == kern, (n, deg)
+    for n, kern in ((32, "k_pcg_resident"), (60, "k_pcg_resident"), (72, "k_pcg_stream"), (96, "k_pcg_stream")):
+        assert bench.mixed_kernel(nodes(n), 13 * nodes(n)) == kern, n
