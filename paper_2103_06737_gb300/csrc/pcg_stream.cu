@@ -17,8 +17,8 @@
 //  - c += alpha p waits for the next product, which reads p anyway, and vector passes move 16
 //    bytes per lane.
 // Measured per Jacobi iteration, against a kernel that read columns and values from global memory
-// with an L2 prefetch one step ahead: edge system of the 64^3 mesh (1.9M rows) 67 -> 50 us, of
-// 96^3 (6.3M rows) 235 -> 189 us (945 MB: 74% of a 6.8 TB/s copy), node system of 96^3 31 -> 25 us.
+// with an L2 prefetch one step ahead: edge system of the 64^3 mesh (1.9M rows) 67 -> 49 us, of
+// 96^3 (6.3M rows) 235 -> 184 us (945 MB: 75% of a 6.8 TB/s copy), node system of 96^3 31 -> 24 us.
 // With only the copies (no gather, no vectors) a 64^3 pass takes 36 us; the rest is the
 // instructions per entry and the gather's latency.  Tried and slower: a ring per warp with
 // its own copies (58 us), two slices per warp at once on 12 warps (67 us), 19 or 23 consumer warps

@@ -214,7 +214,7 @@ __device__ __forceinline__ void warp_run_reduce(int key, Real v[NV], unsigned* h
 // are positive, so the FP32 fraction is within 4 roundings (5e-7) of the exact one, and two that
 // differ by more than 1e-5 of the larger are ordered as in FP64.  Only closer ones are compared in
 // FP64, by cross-multiplication.  (The comparison ran in FP64 for every warp that held one
-// such lane, a fifth of the FP64 issue slots of the walk, which GB300's FP64 pipe bounds.)
+// such lane, a fifth of the walk's FP64 instructions, and GB300's FP64 pipe bounds it.)
 __device__ __forceinline__ int first_exit(const double la[4], const double lb[4], unsigned cand) {
     if ((cand & (cand - 1u)) == 0u) return __ffs(cand) - 1;
     int kx = -1;
