@@ -566,6 +566,7 @@ def run_gpu(args):
     solv = (args.solver.split(",") + args.solver.split(","))[:2]
     code = {"mixed": F.FP_PC_JACOBI, "fp64": F.FP_PC_JACOBI_FP64}
     precond = F.FP_PC_JACOBI
+    pdeg = [1, 1]
     if field:
         F.fem_pic_field_setup(lib.h, wl.dt)
         F.fem_pic_field_options(lib.h, code[solv[0]], code[solv[1]], args.inner_tol)
