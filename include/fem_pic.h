@@ -51,7 +51,7 @@ typedef struct fem_pic fem_pic_t;
 typedef enum {
     FP_OK = 0,
     FP_EINVAL = 1,   /* bad argument, size or pointer; invalid cell id; non-finite particle state */
-    FP_ECUDA = 2,    /* a CUDA runtime call failed (text in fem_pic_last_error) */
+    FP_ECUDA = 2,    /* a CUDA runtime call failed, or a kernel's bounded wait ran out (text in fem_pic_last_error) */
     FP_EWALK = 3,    /* a particle hit the crossing bound of the tet walk */
     FP_ENOCONV = 4,  /* an iterative solve reached its iteration cap, or its residual is no finite number */
     FP_EGEOM = 5     /* a tet with zero volume, or a non-manifold face */
