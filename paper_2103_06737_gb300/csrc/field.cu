@@ -319,6 +319,7 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
     const int ph = system == FP_SYS_NEWMARK ? PH_CG_NEWMARK : PH_CG_GAUSS;
     F->last_fp64[slot] = use64;
     F->slot_sys[slot] = system;
+    F->exchanges[slot] = false;
     if (!use64) {
         const bool nm = system == FP_SYS_NEWMARK;
         const __nv_bfloat16* dl16 = learned_precond(F, system);
@@ -331,7 +332,9 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
         const int max_outer = 12;
         PhaseTimer pt(ctx, ph, s);
         const ResidentPlan& P = F->res[system];
-        if (P.on && (deg <= 1 || P.smem_poly)) {
+        const bool on_chip = P.on && (deg <= 1 || P.smem_poly);
+        F->exchanges[slot] = !(on_chip && P.one);
+        if (on_chip) {
             ResidentArgs a{};
             a.S = nm ? Sell{F->pe_ptr, F->pe_w, F->pe_col} : Sell{F->sn_ptr, F->sn_w, F->sn_col};
             a.val = nm ? F->pe_A : F->sn_L, a.val32 = nm ? F->pe_A32 : F->sn_L32;
@@ -377,10 +380,11 @@ fp_status run_pcg(fem_pic* ctx, int system, const double* rhs, double* x, double
 // tol: the tolerance the solve had (FP_ENOCONV where it missed it); below 0: only the numbers
 fp_status fill_info(fem_pic* ctx, int slot, double tol, fp_solve_info* info, cudaStream_t s, float ms) {
     if (!info) return FP_OK;
-    double o[4];
-    FP_CUDA_TRY(ctx, cudaMemcpyAsync(o, ctx->field->out + 4 * slot, sizeof o, cudaMemcpyDeviceToHost, s));
+    GridReport r;
+    FP_CUDA_TRY(ctx, cudaMemcpyAsync(&r, static_cast<const char*>(ctx->field->sync) + kGridMark, sizeof r,
+                                     cudaMemcpyDeviceToHost, s));
     FP_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    fp_status met = solve_outcome(o, tol, info);
+    fp_status met = solve_outcome(r.out + 4 * slot, r.mark != 0 && ctx->field->exchanges[slot], tol, info);
     if (tol < 0.0 && met == FP_ENOCONV) met = FP_OK;
     if (met == FP_ECUDA) ctx->err = "a field solve gave up waiting for its other blocks: no solution (fem_pic_status resets it)";
     info->ms = ms;
@@ -550,7 +554,9 @@ fp_status launch_exchange_selftest(fem_pic* ctx, double limit_s, cudaStream_t s)
 // after a wait of a mixed solver ran out: the words of its grid exchanges start afresh
 cudaError_t field_reset_sync(fem_pic* ctx, cudaStream_t s) {
     if (!ctx->field || !ctx->field->sync) return cudaSuccess;
-    return cudaMemsetAsync(ctx->field->sync, 0, grid_sync_bytes(ctx->sm_count), s);
+    char* m = static_cast<char*>(ctx->field->sync);
+    const cudaError_t e = cudaMemsetAsync(m, 0, kGridOut, s);   // (not the output words)
+    return e != cudaSuccess ? e : cudaMemsetAsync(m + kGridLine, 0, grid_sync_bytes(ctx->sm_count) - kGridLine, s);
 }
 
 void field_free(fem_pic* ctx) {
@@ -559,7 +565,7 @@ void field_free(fem_pic* ctx) {
     learned_free(F);
     void* ptrs[] = {F->e_rp, F->e_col, F->n_rp, F->n_col, F->Adinv, F->Ldinv,
                     F->edge_fixed, F->node_fixed, F->face_edges, F->r, F->z, F->p, F->q, F->rhs, F->tmp,
-                    F->delta, F->qd, F->red, F->out, F->Ldinv32, F->r32,
+                    F->delta, F->qd, F->red, F->Ldinv32, F->r32,
                     F->z32, F->p32, F->q32, F->c32, F->s32, F->d32[0], F->d32[1], F->se_d16, F->sn_d16, F->pe_ptr, F->pe_w, F->pe_col, F->perm_e, F->pe_A, F->pe_A32, F->pe_dinv32, F->pb, F->px, F->alpha, F->msum, F->se_ptr, F->se_w, F->se_col, F->sn_ptr, F->sn_w,
                     F->sn_col, F->se_M, F->se_S, F->se_A, F->sn_L, F->sn_L32, F->sync, F->res[0].pp, F->res[1].pp};
     for (void* p : ptrs)
@@ -860,12 +866,11 @@ static fp_status field_setup(fem_pic_t* ctx, double dt, double eps, double mu, i
     if (st == FP_OK) {
         FP_CUDA_TRY(ctx, cudaMalloc(&F->sync, grid_sync_bytes(ctx->sm_count)));
         FP_CUDA_TRY(ctx, cudaMemset(F->sync, 0, grid_sync_bytes(ctx->sm_count)));
+        F->out = reinterpret_cast<double*>(static_cast<char*>(F->sync) + kGridOut);
     }
     if (st == FP_OK) {
         F->grid = std::max(F->grid_e, F->grid_n);
         FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->red, 9 * (size_t)F->grid * sizeof(double)));
-        FP_CUDA_TRY(ctx, cudaMalloc((void**)&F->out, 16 * sizeof(double)));
-        FP_CUDA_TRY(ctx, cudaMemset(F->out, 0, 16 * sizeof(double)));
     }
     if (st == FP_OK && bc == FP_BC_NEUMANN) {
         std::vector<double> a(hc.nn);

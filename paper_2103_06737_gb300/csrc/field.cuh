@@ -36,12 +36,14 @@ __host__ __device__ inline bool solve_met(double rr, double thr) { return rr <= 
 // What a solve's output words (iterations, |r|^2, |reference|^2, refinements) say: the numbers of info,
 // and FP_OK, or FP_ENOCONV where the relative residual is not within tol (NaN included).  FP_ECUDA
 // where the refinements still are kAbandoned: a mixed solver writes {0, infinity, 1, kAbandoned} when
-// it starts, so that one that gives up does not leave an earlier solve's numbers.
+// it starts, so that one that gives up does not leave an earlier solve's numbers.  marked: an exchange
+// of the handle was abandoned; FP_ECUDA too, since a block can give up on a last exchange that the
+// others see complete, and its rows of the solution are then missing.
 constexpr double kAbandoned = -1.0;
 __host__ __device__ inline void solve_begin(double out[4]) {
     out[0] = 0.0, out[1] = HUGE_VAL, out[2] = 1.0, out[3] = kAbandoned;
 }
-fp_status solve_outcome(const double out[4], double tol, fp_solve_info* info);
+fp_status solve_outcome(const double out[4], bool marked, double tol, fp_solve_info* info);
 
 // launch shape of the on-chip mixed solver for one system (pcg_resident.cu)
 struct ResidentPlan {
@@ -104,11 +106,12 @@ struct FieldDev {
     int64_t sectors_e[2] = {0, 0};  // gathered 32-byte sectors per product: edge order, solver order
     std::vector<int32_t> hwidth[2];  // host copies of the SELL slice widths (Newmark, Gauss)
     double* red = nullptr;          // reduction partials
-    double* out = nullptr;          // [8] solver outputs (iterations, rr, bb) of the last two solves
+    double* out = nullptr;          // [8] output words of the last two solves (in sync's memory)
     int grid = 0;                   // co-resident blocks (cooperative launch limit)
     int grid_e = 0, grid_n = 0;     // grids of the edge and node systems
     int bs_e = 256, bs_n = 256;     // and their block sizes
     int last_fp64[2] = {0, 0};      // solver used by the last solve in each info slot
+    bool exchanges[2] = {false, false};   // whether its blocks exchanged through memory
     ResidentPlan res[2];            // on-chip solver, Newmark and Gauss systems
     StreamPlan stream[2];           // streamed solver, Newmark and Gauss systems
     void* sync = nullptr;           // words of the mixed solvers' grid exchanges (grid_sync.cuh)

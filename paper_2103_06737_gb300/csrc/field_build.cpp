@@ -13,10 +13,10 @@
 
 namespace fempic {
 
-fp_status solve_outcome(const double out[4], double tol, fp_solve_info* info) {
-    const bool abandoned = out[3] == kAbandoned;
+fp_status solve_outcome(const double out[4], bool marked, double tol, fp_solve_info* info) {
+    const bool begun = out[3] == kAbandoned, abandoned = begun || marked;
     info->iters = (int32_t)out[0];
-    info->outer = abandoned ? 0 : (int32_t)out[3];
+    info->outer = begun ? 0 : (int32_t)out[3];
     info->rel_res = out[2] > 0 ? std::sqrt(out[1] / out[2]) : std::sqrt(out[1]);
     info->abs_res = std::sqrt(out[1]);
     return abandoned ? FP_ECUDA : info->rel_res <= tol ? FP_OK : FP_ENOCONV;

@@ -28,6 +28,7 @@
 #pragma once
 
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 
 #include "internal.cuh"
@@ -40,10 +41,17 @@ namespace fempic {
 // Limit of a wait.  A launch's first exchange also waits for blocks that have not started because a
 // kernel of another stream still holds their SMs (30 s); the later ones only for blocks at work (2 s).
 constexpr uint64_t kGridStartNs = 30000000000ull, kGridWaitNs = 2000000000ull;
-// device memory of one handle's exchanges (zeroed at setup): the words at rest and the mark of an
-// abandoned exchange, the words in use (two exchanges; a line each), then the blocks' partials for
-// the sums that are added one by one (two copies of three doubles per block)
-constexpr size_t kGridLine = 128, kGridMark = 32;
+// device memory of one handle's exchanges (zeroed at setup): the words at rest, the mark of an
+// abandoned exchange and the solves' output words, read with it by one copy (GridReport); the words
+// in use (two exchanges; a line each), then the blocks' partials for the sums that are added one by
+// one (two copies of three doubles per block)
+constexpr size_t kGridLine = 128, kGridMark = 32, kGridOut = 64;
+struct GridReport {
+    unsigned long long mark, pad[3];
+    double out[8];               // four per info slot
+};
+static_assert(sizeof(GridReport) == kGridLine - kGridMark && offsetof(GridReport, out) == kGridOut - kGridMark,
+              "GridReport layout");
 constexpr int kFail = 4;
 inline size_t grid_sync_bytes(int blocks) { return 3 * kGridLine + (size_t)2 * blocks * 3 * 8; }
 

@@ -9,9 +9,9 @@ using namespace fempic;
 extern "C" {
 
 // the status and {rel_res, abs_res, iters, outer} that a solve's output words stand for
-int hs_outcome(const double* out, double tol, double* r) {
+int hs_outcome(const double* out, int marked, double tol, double* r) {
     fp_solve_info info{};
-    const int st = (int)solve_outcome(out, tol, &info);
+    const int st = (int)solve_outcome(out, marked != 0, tol, &info);
     r[0] = info.rel_res, r[1] = info.abs_res, r[2] = info.iters, r[3] = info.outer;
     return st;
 }

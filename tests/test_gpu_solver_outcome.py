@@ -59,7 +59,10 @@ def test_abandoned_exchange_is_reported_and_reset(n):
     x0 = vec(lib.n_edges)
     st, info = solve(x0)
     assert st == F.FP_OK and info["iters"] > 0
+    assert F.fem_pic_field_last_info(lib.h)[0]["iters"] == info["iters"]
     F.fem_pic_selftest_wait(lib.h, 1e-3)
+    with pytest.raises(F.FemPicError, match="gave up waiting"):
+        F.fem_pic_field_last_info(lib.h)       # good output words beside the mark are not taken either
     with pytest.raises(F.FemPicError, match="gave up waiting"):
         solve(vec(lib.n_edges))
     solve(vec(lib.n_edges), info=False)
@@ -95,4 +98,23 @@ def test_failed_learned_init_leaves_no_network(model):
     if model == F.FP_LEARNED_PRECOND:
         F.fem_pic_learned_build(lib.h)
     assert step(F.FP_PC_LEARNED)[0] == F.FP_OK and lib.status() == F.FP_OK
+    lib.close()
+
+
+def test_solvers_without_exchanges_work_beside_the_mark():
+    """A system of one block and the FP64 solver exchange nothing through the words: they go on."""
+    lib = _lib(9)
+    rhs = torch.zeros(lib.n_edges, dtype=torch.float64, device="cuda")
+    rp, _, _ = F.fem_pic_field_matrix(lib.h, 2)
+    rhs[int(np.nonzero(np.diff(rp) > 1)[0][0])] = 1.0
+    F.fem_pic_selftest_wait(lib.h, 1e-3)
+    x = torch.zeros_like(rhs)
+    st, info = F.fem_pic_field_solve(lib.h, F.FP_SYS_NEWMARK, rhs, x, tol=1e-10, precond=F.FP_PC_JACOBI_FP64)
+    assert st == F.FP_OK and info["rel_res"] <= 1e-10
+    g = torch.zeros(lib.n_nodes, dtype=torch.float64, device="cuda")     # 1,000 nodes: one block
+    rp, _, _ = F.fem_pic_field_matrix(lib.h, 3)
+    g[int(np.nonzero(np.diff(rp) > 1)[0][0])] = 1.0
+    st, info = F.fem_pic_field_solve(lib.h, F.FP_SYS_GAUSS, g, torch.zeros_like(g), tol=1e-10)
+    assert st == F.FP_OK and info["rel_res"] <= 1e-10
+    assert lib.status() == F.FP_ECUDA and lib.status() == F.FP_OK
     lib.close()

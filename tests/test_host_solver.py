@@ -24,7 +24,7 @@ def hs(tmp_path_factory):
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(out)
-    lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
+    lib.hs_outcome.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_double, ctypes.c_void_p]
     lib.hs_segments.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_void_p]
     lib.hs_word_sum.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_float, ctypes.c_void_p]
     lib.hs_wait_seconds.restype = ctypes.c_double
@@ -41,10 +41,12 @@ def hs(tmp_path_factory):
     ((0, INF, 1.0, -1), ECUDA)])                                    # as a solve writes them when it starts
 def test_outcome_of_a_solve(hs, words, status):
     w, r = np.array(words, np.float64), np.zeros(4)
-    assert hs.hs_outcome(w.ctypes.data, 1e-10, r.ctypes.data) == status
+    assert hs.hs_outcome(w.ctypes.data, 0, 1e-10, r.ctypes.data) == status
     assert (r[2], r[3]) == (words[0], max(words[3], 0))
     # the device sets the status word's bit by the same rule
     assert hs.hs_met(w[1], 1e-20 * w[2]) == (status == OK)
+    # whatever they say, an exchange was abandoned: a block may have left without its rows
+    assert hs.hs_outcome(w.ctypes.data, 1, 1e-10, r.ctypes.data) == ECUDA
 
 
 def test_first_exchange_waits_for_blocks_that_start_late(hs):
