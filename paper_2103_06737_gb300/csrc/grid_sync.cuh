@@ -142,6 +142,9 @@ struct GridSync {
     template <int NW>
     __device__ __forceinline__ bool arrive_wait(int par, const unsigned long long (&q)[NW], unsigned long long (&d)[NW]) {
         unsigned long long* w = word(par);
+        unsigned long long p[NW];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) p[k] = sh->rest[2 * par + k];
         // the last addition releases, the load of that word acquires
 #pragma unroll
         for (int k = 1; k < NW; ++k)
@@ -159,7 +162,7 @@ struct GridSync {
             asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(c[0]) : "l"(w) : "memory");
 #pragma unroll
             for (int k = 0; k < NW; ++k) {
-                d[k] = c[k] - sh->rest[2 * par + k];
+                d[k] = c[k] - p[k];
                 all = all && (int)(d[k] & 255ull) == nb;
             }
             if (all) {
@@ -208,6 +211,7 @@ struct GridSync {
 #pragma unroll
             for (int k = 0; k < NV; ++k) sh->part[par][k][wid] = v[k];
         __syncthreads();
+        const bool alive = ONE || sh->rest[kFail] == 0;   // early: its latency beside the shuffles'
         if (ONE || wid == 0) {
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
@@ -227,7 +231,7 @@ struct GridSync {
                 q[k] = word_put(v[k], e[k]);
                 parts[k * nb + blockIdx.x] = v[k];             // for the sums added one by one
             }
-            const bool ok = sh->rest[kFail] == 0 && arrive_wait<NV>(par, q, d);
+            const bool ok = alive && arrive_wait<NV>(par, q, d);
             bool exact = false;
 #pragma unroll
             for (int k = 0; k < NV; ++k) exact = !word_total(d[k], e[k], &sh->tot[par][k]) || exact;
