@@ -17,8 +17,8 @@
 // Bound by latency: per Jacobi iteration two exchanges (1.5 us each on 152 blocks), one product
 // (about 1 us for one slice a warp, 4 us for two slices a warp of the edge system).  Measured on
 // the 32^3 mesh, per solve, against a kernel with the same operator in shared memory, vectors in
-// global memory and cooperative-groups barriers: edge system 565 -> 354 us (17 iterations of degree
-// 3), node system 253 -> 179 us (7 of degree 8); 4^3 mesh (one block) 141 -> 59 us and 52 -> 19 us.
+// global memory and cooperative-groups barriers: edge system 565 -> 352 us (17 iterations of degree
+// 3), node system 253 -> 175 us (7 of degree 8); 4^3 mesh (one block) 141 -> 59 us and 52 -> 19 us.
 // Two or three rows a lane in registers instead of shared memory spilled at the 80 registers that
 // 800 threads leave; vectors in shared memory cost no time that shows.
 #include <algorithm>
